@@ -168,7 +168,8 @@ struct Smem {
     const float *sig_a, *cdf, *maj, *inv_maj, *qy;
     unsigned long long *tal;   // shared memory, or the launch's global tallies (tal_global)
     unsigned long long *cnt;
-    bool tal_global;
+    uint32_t *cnt32;           // 32-bit counters of the persistent forms (cnt_add)
+    bool tal_global, persistent;
 };
 
 // Frequent counters live in registers; the rest go straight to shared memory.
@@ -176,12 +177,41 @@ struct RegCnt {
     uint32_t steps, nulls, events, scatters, connections, connect_steps, cell_walks;
 };
 
-// Adds one per calling lane. The lanes that arrive together add once, through their lowest lane,
-// instead of queueing on one shared-memory word.
+// Adds one per calling lane. The persistent forms count in 32 bits, one native shared-memory addition
+// (a 64-bit one is a loop, and adding up the lanes first cost 24 instructions at each of some
+// twenty sites: code that the instruction cache has to hold); counters_carry moves the counts on long
+// before they can wrap. The one-thread-per-path forms, whose path may run for as long as its step
+// budget lets it, add the lanes that arrive together through their lowest lane in 64 bits.
 __device__ __forceinline__ void cnt_add(const Smem &sm, int k)
 {
+    if (sm.persistent) {
+        atomicAdd(&sm.cnt32[k], 1u);
+        return;
+    }
     const unsigned mask = __activemask();
     if ((threadIdx.x & 31) == __ffs(mask) - 1) atomicAdd(&sm.cnt[k], (unsigned long long)__popc(mask));
+}
+
+// The same for a counter that differs between the lanes.
+__device__ __forceinline__ void cnt_add_any(const Smem &sm, int k)
+{
+    if (sm.persistent) atomicAdd(&sm.cnt32[k], 1u);
+    else atomicAdd(&sm.cnt[k], 1ull);
+}
+
+// Called by every warp of a persistent form once in CARRY_ROUNDS of its rounds. A round makes at most
+// MAX_REGROUP steps a lane and a step adds at most twice to one counter, so between two calls the
+// (at most eight) warps of a block add less than 2^30.
+constexpr int MAX_REGROUP = 64;
+constexpr uint32_t CARRY_ROUNDS = 1u << 14;
+__device__ __forceinline__ void counters_carry(const Smem &sm)
+{
+    const int lane = threadIdx.x & 31;
+    if (lane < FLR_NCOUNTERS) {
+        const uint32_t v = atomicExch(&sm.cnt32[lane], 0u);
+        if (v) atomicAdd(&sm.cnt[lane], (unsigned long long)v);
+    }
+    __syncwarp();
 }
 
 __device__ __forceinline__ void tally_add(const Smem &sm, int idx, float w)
@@ -410,11 +440,10 @@ __device__ __forceinline__ Coeffs coeffs_at(const M &m, float3 x, int b)
     const float cc[4] = {c.x, c.y, c.z, c.w};
     const float4 sa = m.sig_a4(b);
     const float ss[4] = {sa.x, sa.y, sa.z, sa.w};
-    const int D = m.D();
 #pragma unroll
     for (int d = 0; d < MAXD; ++d) {
-        k.dye[d] = (d < D) ? ss[d] * cc[d] : 0.0f;
-        k.total += k.dye[d];
+        k.dye[d] = __fmul_rn(ss[d], cc[d]);   // 0 for d >= D: both tables are zero there
+        k.total = __fadd_rn(k.total, k.dye[d]);
     }
     return k;
 }
@@ -435,11 +464,11 @@ __device__ __forceinline__ float exit_distance(const M &m, float3 x, float3 w, f
     const float xs[3] = {x.x, x.y, x.z}, ws[3] = {w.x, w.y, w.z}, is[3] = {iw.x, iw.y, iw.z};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        if (ws[k] == 0.0f) continue;
         const bool pos = ws[k] > 0.0f;
-        float t = ((pos ? m.hi(k) : m.lo(k)) - xs[k]) * is[k];
-        t = fmaxf(t, 0.0f);
-        if (t < best) { best = t; face = 2 * k + (pos ? 1 : 0); }
+        const float t = fmaxf(((pos ? m.hi(k) : m.lo(k)) - xs[k]) * is[k], 0.0f);
+        const bool nearer = ws[k] != 0.0f && t < best;   // selects, no branches
+        best = nearer ? t : best;
+        face = nearer ? 2 * k + (pos ? 1 : 0) : face;
     }
     return best;
 }
@@ -453,13 +482,23 @@ __device__ __forceinline__ float sqrt_approx(float x)
     return r;
 }
 
+// The hardware's approximate reciprocal (PTX rcp.approx.ftz.f32, 1 ulp). The same bits as
+// __fdividef(1, x) for every normal x whose reciprocal is normal, without the range checks that
+// surround it (3 instructions instead of 10).
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // Componentwise inverse of a direction (0 for a zero component). The approximate reciprocal
-// (2 ulp) is plenty for distances to planes and cost 7 % less time per Cornell-box step than the
+// is plenty for distances to planes and cost 7 % less time per Cornell-box step than the
 // correctly rounded one.
 __device__ __forceinline__ float3 inv_dir(float3 w)
 {
-    return make_float3(w.x != 0.0f ? __fdividef(1.0f, w.x) : 0.0f, w.y != 0.0f ? __fdividef(1.0f, w.y) : 0.0f,
-                       w.z != 0.0f ? __fdividef(1.0f, w.z) : 0.0f);
+    return make_float3(w.x != 0.0f ? rcp_approx(w.x) : 0.0f, w.y != 0.0f ? rcp_approx(w.y) : 0.0f,
+                       w.z != 0.0f ? rcp_approx(w.z) : 0.0f);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1039,16 +1078,15 @@ struct NoObs {
 };
 
 // One tracking step (null or real collision, wall bounce or escape). Returns the connection the
-// step asks for, if any.
-template <class M, class Obs = NoObs>
-__device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Smem &sm, Path &p,
-                                           RegCnt &rc, const Obs &obs = Obs())
+// step asks for, if any; a step that ends the path says which counter it ends on in `end`.
+template <class M, class Obs>
+__device__ __forceinline__ Conn track_body(const M &m, const RunDev &R, const Smem &sm, Path &p,
+                                           RegCnt &rc, const Obs &obs, int &end)
 {
     Conn c;
     c.valid = false;
     if ((long long)p.step >= R.max_steps) {
-        cnt_add(sm, FLR_C_STEP_BUDGET);
-        finish(R, p);
+        end = FLR_C_STEP_BUDGET;
         return c;
     }
     rc.steps++;
@@ -1076,8 +1114,7 @@ __device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Sm
     if (tf >= te) {
         p.x = make_float3(p.x.x + te * p.w.x, p.x.y + te * p.w.y, p.x.z + te * p.w.z);
         if (face < 0) {  // no direction component: cannot happen for unit directions
-            cnt_add(sm, FLR_C_NONFINITE);
-            finish(R, p);
+            end = FLR_C_NONFINITE;
             return c;
         }
         if (!(m.wall_mask() & (1 << face))) {
@@ -1088,7 +1125,7 @@ __device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Sm
                 float ct;
                 const float F = fresnel_refl(fabsf(comp(p.w, k)), m.ior(), ct);
                 if (b0.b < F) {
-                    if (p.n_events == R.max_events) { cnt_add(sm, FLR_C_CAP_HITS); finish(R, p); return c; }
+                    if (p.n_events == R.max_events) { end = FLR_C_CAP_HITS; return c; }
                     p.n_events++;
                     rc.events++;
                     cnt_add(sm, FLR_C_IFACE_REFLECTIONS);
@@ -1097,28 +1134,27 @@ __device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Sm
                     p.iw = inv_dir(p.w);
                     if (p.n_events >= R.n_rr) {
                         const float q = fminf(p.wt, 1.0f);
-                        if (!(b1.c < q)) { cnt_add(sm, FLR_C_RR_KILLS); finish(R, p); return c; }
+                        if (!(b1.c < q)) { end = FLR_C_RR_KILLS; return c; }
                         p.wt = p.wt < 1.0f ? 1.0f : p.wt;
                     }
                     return c;
                 }
             }
             m.tally(tal_face(m.B()) + (p.fl * 6 + face) * m.B() + p.bin, p.wt);
-            cnt_add(sm, FLR_C_ESCAPES);
-            finish(R, p);
+            end = FLR_C_ESCAPES;
             return c;
         }
         // the paper's model drops excitation light reflected by a wall before any emission
-        if (R.paper_mode && !p.fl) { cnt_add(sm, FLR_C_VF_REJECTED); finish(R, p); return c; }
-        if (p.n_events == R.max_events) { cnt_add(sm, FLR_C_CAP_HITS); finish(R, p); return c; }
+        if (R.paper_mode && !p.fl) { end = FLR_C_VF_REJECTED; return c; }
+        if (p.n_events == R.max_events) { end = FLR_C_CAP_HITS; return c; }
         p.n_events++;
         rc.events++;
         cnt_add(sm, FLR_C_WALL_BOUNCES);
         if (R.analog) {
-            if (!(b1.d < m.wall_albedo())) { cnt_add(sm, FLR_C_ABSORBED_DEAD); finish(R, p); return c; }
+            if (!(b1.d < m.wall_albedo())) { end = FLR_C_ABSORBED_DEAD; return c; }
         } else {
             p.wt *= m.wall_albedo();
-            if (p.wt == 0.0f) { cnt_add(sm, FLR_C_ABSORBED_DEAD); finish(R, p); return c; }
+            if (p.wt == 0.0f) { end = FLR_C_ABSORBED_DEAD; return c; }
         }
         dax = face >> 1;
         dsg = (face & 1) ? -1.0f : 1.0f;
@@ -1144,7 +1180,7 @@ __device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Sm
             if (b1.a < g) {
                 p.w = phong_dir(du1, du2, r, e);
                 const float co = dsg * comp(p.w, dax);
-                if (!(co > 0.0f)) { cnt_add(sm, FLR_C_ABSORBED_DEAD); finish(R, p); return c; }
+                if (!(co > 0.0f)) { end = FLR_C_ABSORBED_DEAD; return c; }
                 p.wt *= (e + 2.0f) / (e + 1.0f) * co;
                 gw = 2;
             }
@@ -1175,7 +1211,7 @@ __device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Sm
                 return c;
             }
         }
-        if (p.n_events == R.max_events) { cnt_add(sm, FLR_C_CAP_HITS); finish(R, p); return c; }
+        if (p.n_events == R.max_events) { end = FLR_C_CAP_HITS; return c; }
         p.n_events++;
         rc.events++;
         // particle type in proportion to its coefficient (Sec. 4.1)
@@ -1199,20 +1235,19 @@ __device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Sm
         if (ev < 0) {
             rc.scatters++;
             // the paper's model drops scattered excitation light (Sec. 4.1)
-            if (R.paper_mode && !p.fl) { cnt_add(sm, FLR_C_VF_REJECTED); finish(R, p); return c; }
+            if (R.paper_mode && !p.fl) { end = FLR_C_VF_REJECTED; return c; }
         } else if (ev < D) {
             cnt_add(sm, FLR_C_DYE_ABSORPTIONS);
             m.tally(tal_absorbed(m.B()) + ev * m.B() + p.bin, p.wt);
             if ((R.max_inelastic >= 0 && p.n_inel >= R.max_inelastic) || (R.paper_mode && p.n_inel >= 1)) {
-                cnt_add(sm, FLR_C_VF_REJECTED);
-                finish(R, p);
+                end = FLR_C_VF_REJECTED;
                 return c;
             }
             if (R.analog) {
-                if (!(b1.d < m.qy(ev))) { cnt_add(sm, FLR_C_ABSORBED_DEAD); finish(R, p); return c; }
+                if (!(b1.d < m.qy(ev))) { end = FLR_C_ABSORBED_DEAD; return c; }
             } else {
                 p.wt *= m.qy(ev);
-                if (p.wt == 0.0f) { cnt_add(sm, FLR_C_ABSORBED_DEAD); finish(R, p); return c; }
+                if (p.wt == 0.0f) { end = FLR_C_ABSORBED_DEAD; return c; }
             }
             p.bin = sample_cdf(m.cdf(ev), m.B(), b1.b);
             m.tally(tal_emitted(m.B()) + ev * m.B() + p.bin, p.wt);
@@ -1221,8 +1256,7 @@ __device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Sm
             p.fl = 1;
         } else {
             m.tally(tal_absorbed(m.B()) + D * m.B() + p.bin, p.wt);
-            cnt_add(sm, FLR_C_ABSORBED_DEAD);
-            finish(R, p);
+            end = FLR_C_ABSORBED_DEAD;
             return c;
         }
     }
@@ -1248,13 +1282,34 @@ __device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Sm
     if (m.sensor() && gw == 0) c = Conn{p.x, p.wt, p.bin, dax < 0 ? -1 : 2 * dax + (dsg > 0.0f ? 1 : 0), p.pid, step, true};
     if (p.n_events >= R.n_rr) {
         const float q = fminf(p.wt, 1.0f);
-        if (!(b1.c < q)) { cnt_add(sm, FLR_C_RR_KILLS); finish(R, p); return c; }
+        if (!(b1.c < q)) { end = FLR_C_RR_KILLS; return c; }
         p.wt = p.wt < 1.0f ? 1.0f : p.wt;   // w / min(w, 1), exactly
     }
     if (!(isfinite(p.wt) && isfinite(p.x.x) && isfinite(p.x.y) && isfinite(p.x.z))) {
-        cnt_add(sm, FLR_C_NONFINITE);
-        finish(R, p);
+        end = FLR_C_NONFINITE;
         c.valid = false;
+    }
+    return c;
+}
+
+// The step with its end: the count and the path's event record stand once, behind the step, instead
+// of at each of the fourteen places where a path can end. What bounds the persistent kernels is the
+// instruction cache: at five warps a scheduler more warps only raise the stalls for want of an
+// instruction (0.55 to 3.6 per instruction at eight), and a kernel of more phases than tracking and
+// drain loses more to them than its fuller lanes gain. So the loops' code is kept small: this, the
+// counters of cnt_add, the selects of exit_distance and the reciprocals of inv_dir took the step
+// from 1,460 to 860 instructions, and (per call, on the current sizes) the Cornell box from 11.07 to
+// 10.08 ms, with four hero wavelengths (8 paths a pixel) from 11.31 to 8.58 ms, the light sheet from 205 to
+// 189 ms, 256 batched media from 41.3 to 37.8 ms, the camera view from 0.84 to 0.76 ms.
+template <class M, class Obs = NoObs>
+__device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Smem &sm, Path &p,
+                                           RegCnt &rc, const Obs &obs = Obs())
+{
+    int end = -1;
+    const Conn c = track_body(m, R, sm, p, rc, obs, end);
+    if (end >= 0) {
+        cnt_add_any(sm, end);
+        finish(R, p);
     }
     return c;
 }
@@ -1305,7 +1360,7 @@ __host__ __device__ inline SmemLayout smem_layout(int B, int form, int block)
     L.tal_global = form == FLR_FORM_WAVEFRONT_WARP || form == FLR_FORM_WAVEFRONT_POOL;
     if (!L.tal_global) off += tal_size(B) * 8;
     L.cnt_off_bytes = off;
-    off += FLR_NCOUNTERS * 8;
+    off += FLR_NCOUNTERS * 12;
     off = ((off + 15) / 16) * 16;
     L.queue_off_bytes = off;
     if (form == FLR_FORM_WAVEFRONT) off += 2 * block * 32 + 16;
@@ -1316,7 +1371,7 @@ __host__ __device__ inline SmemLayout smem_layout(int B, int form, int block)
 }
 
 __device__ __forceinline__ Smem block_prologue(const SceneDev &S, unsigned char *raw, const SmemLayout &L,
-                                               unsigned long long *global_tal)
+                                               unsigned long long *global_tal, bool persistent = false)
 {
     float *tab = reinterpret_cast<float *>(raw);
     for (int i = threadIdx.x; i < L.tab_floats; i += blockDim.x) tab[i] = S.tables[i];
@@ -1325,9 +1380,15 @@ __device__ __forceinline__ Smem block_prologue(const SceneDev &S, unsigned char 
     if (!L.tal_global)
         for (int i = threadIdx.x; i < tal_size(S.B); i += blockDim.x) tal[i] = 0ull;
     unsigned long long *cnt = reinterpret_cast<unsigned long long *>(raw + L.cnt_off_bytes);
-    for (int i = threadIdx.x; i < FLR_NCOUNTERS; i += blockDim.x) cnt[i] = 0ull;
+    uint32_t *cnt32 = reinterpret_cast<uint32_t *>(cnt + FLR_NCOUNTERS);
+    for (int i = threadIdx.x; i < FLR_NCOUNTERS; i += blockDim.x) {
+        cnt[i] = 0ull;
+        cnt32[i] = 0u;
+    }
     __syncthreads();
     Smem sm;
+    sm.cnt32 = cnt32;
+    sm.persistent = persistent;
     sm.sig_a = tab + tab_sig_a(S.B);
     sm.cdf = tab + tab_cdf(S.B);
     sm.maj = tab + tab_majorant(S.B);
@@ -1339,11 +1400,18 @@ __device__ __forceinline__ Smem block_prologue(const SceneDev &S, unsigned char 
     return sm;
 }
 
+// A counter of the block once its warps are done.
+__device__ __forceinline__ unsigned long long cnt_total(const Smem &sm, int k)
+{
+    return sm.cnt[k] + (sm.persistent ? sm.cnt32[k] : 0u);
+}
+
 // Sets the launch's error word when a path or a connection of this block ran out of its step
 // budget (flr_status then reports FLR_ERR_BUDGET). Called by every thread after a block barrier.
 __device__ __forceinline__ void budget_flag(const RunDev &R, const Smem &sm)
 {
-    if (threadIdx.x == 0 && R.error_word && (sm.cnt[FLR_C_STEP_BUDGET] | sm.cnt[FLR_C_CONNECT_BUDGET]))
+    if (threadIdx.x == 0 && R.error_word &&
+        (cnt_total(sm, FLR_C_STEP_BUDGET) | cnt_total(sm, FLR_C_CONNECT_BUDGET)))
         atomicOr(R.error_word, 1);
 }
 
@@ -1368,7 +1436,7 @@ __device__ __forceinline__ void block_epilogue(const SceneDev &S, const RunDev &
         for (int i = threadIdx.x; i < tal_size(S.B); i += blockDim.x)
             if (sm.tal[i]) atomicAdd(&R.tallies[i], sm.tal[i]);
     for (int i = threadIdx.x; i < FLR_NCOUNTERS; i += blockDim.x)
-        if (sm.cnt[i]) atomicAdd(&R.counters[i], sm.cnt[i]);
+        if (cnt_total(sm, i)) atomicAdd(&R.counters[i], cnt_total(sm, i));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1452,11 +1520,10 @@ __device__ __forceinline__ Coeffs coeffs_of(const M &m, const MatterPt &pt, int 
     const float cc[4] = {pt.c.x, pt.c.y, pt.c.z, pt.c.w};
     const float4 sa = m.sig_a4(b);
     const float ss[4] = {sa.x, sa.y, sa.z, sa.w};
-    const int D = m.D();
 #pragma unroll
     for (int d = 0; d < MAXD; ++d) {
-        k.dye[d] = (d < D) ? ss[d] * cc[d] : 0.0f;
-        k.total += k.dye[d];
+        k.dye[d] = __fmul_rn(ss[d], cc[d]);   // 0 for d >= D: both tables are zero there
+        k.total = __fadd_rn(k.total, k.dye[d]);
     }
     return k;
 }
@@ -1617,14 +1684,13 @@ __device__ __forceinline__ void hero_tally(const M &m, int row, const HeroSet &h
 // One tracking step of a hero path: the single-wavelength step (track_step) with the set's
 // majorant, the weights re-balanced at null collisions and the tallies split among the members.
 template <class M>
-__device__ __forceinline__ Conn track_step_hero(const M &m, const RunDev &R, const Smem &sm, Path &p,
-                                                HeroSet &h, RegCnt &rc)
+__device__ __forceinline__ Conn track_body_hero(const M &m, const RunDev &R, const Smem &sm, Path &p,
+                                                HeroSet &h, RegCnt &rc, int &end)
 {
     Conn c;
     c.valid = false;
     if ((long long)p.step >= R.max_steps) {
-        cnt_add(sm, FLR_C_STEP_BUDGET);
-        finish(R, p);
+        end = FLR_C_STEP_BUDGET;
         return c;
     }
     rc.steps++;
@@ -1641,25 +1707,23 @@ __device__ __forceinline__ Conn track_step_hero(const M &m, const RunDev &R, con
     if (tf >= te) {
         p.x = make_float3(p.x.x + te * p.w.x, p.x.y + te * p.w.y, p.x.z + te * p.w.z);
         if (face < 0) {
-            cnt_add(sm, FLR_C_NONFINITE);
-            finish(R, p);
+            end = FLR_C_NONFINITE;
             return c;
         }
         if (!(m.wall_mask() & (1 << face))) {
             hero_tally(m, tal_face(m.B()) + (p.fl * 6 + face) * m.B(), h, p.wt);
-            cnt_add(sm, FLR_C_ESCAPES);
-            finish(R, p);
+            end = FLR_C_ESCAPES;
             return c;
         }
-        if (p.n_events == R.max_events) { cnt_add(sm, FLR_C_CAP_HITS); finish(R, p); return c; }
+        if (p.n_events == R.max_events) { end = FLR_C_CAP_HITS; return c; }
         p.n_events++;
         rc.events++;
         cnt_add(sm, FLR_C_WALL_BOUNCES);
         if (R.analog) {
-            if (!(b1.d < m.wall_albedo())) { cnt_add(sm, FLR_C_ABSORBED_DEAD); finish(R, p); return c; }
+            if (!(b1.d < m.wall_albedo())) { end = FLR_C_ABSORBED_DEAD; return c; }
         } else {
             p.wt *= m.wall_albedo();
-            if (p.wt == 0.0f) { cnt_add(sm, FLR_C_ABSORBED_DEAD); finish(R, p); return c; }
+            if (p.wt == 0.0f) { end = FLR_C_ABSORBED_DEAD; return c; }
         }
         dax = face >> 1;
         dsg = (face & 1) ? -1.0f : 1.0f;
@@ -1703,7 +1767,7 @@ __device__ __forceinline__ Conn track_step_hero(const M &m, const RunDev &R, con
             }
             return c;
         }
-        if (p.n_events == R.max_events) { cnt_add(sm, FLR_C_CAP_HITS); finish(R, p); return c; }
+        if (p.n_events == R.max_events) { end = FLR_C_CAP_HITS; return c; }
         p.n_events++;
         rc.events++;
         const float ue = b0.c * k.total;
@@ -1746,15 +1810,14 @@ __device__ __forceinline__ Conn track_step_hero(const M &m, const RunDev &R, con
                 hero_tally(m, tal_absorbed(m.B()) + ev * m.B(), ha, p.wt);
             }
             if (R.max_inelastic >= 0 && p.n_inel >= R.max_inelastic) {
-                cnt_add(sm, FLR_C_VF_REJECTED);
-                finish(R, p);
+                end = FLR_C_VF_REJECTED;
                 return c;
             }
             if (R.analog) {
-                if (!(b1.d < m.qy(ev))) { cnt_add(sm, FLR_C_ABSORBED_DEAD); finish(R, p); return c; }
+                if (!(b1.d < m.qy(ev))) { end = FLR_C_ABSORBED_DEAD; return c; }
             } else {
                 p.wt *= m.qy(ev);
-                if (p.wt == 0.0f) { cnt_add(sm, FLR_C_ABSORBED_DEAD); finish(R, p); return c; }
+                if (p.wt == 0.0f) { end = FLR_C_ABSORBED_DEAD; return c; }
             }
             p.bin = sample_cdf(m.cdf(ev), m.B(), b1.b);
             hero_emission(m, ev, p.bin, R.hero, h);
@@ -1764,8 +1827,7 @@ __device__ __forceinline__ Conn track_step_hero(const M &m, const RunDev &R, con
             p.fl = 1;
         } else {
             hero_tally(m, tal_absorbed(m.B()) + D * m.B(), h, p.wt);
-            cnt_add(sm, FLR_C_ABSORBED_DEAD);
-            finish(R, p);
+            end = FLR_C_ABSORBED_DEAD;
             return c;
         }
     }
@@ -1788,13 +1850,25 @@ __device__ __forceinline__ Conn track_step_hero(const M &m, const RunDev &R, con
     if (m.sensor()) c = Conn{p.x, p.wt, p.bin, dax < 0 ? -1 : 2 * dax + (dsg > 0.0f ? 1 : 0), p.pid, step, true};
     if (p.n_events >= R.n_rr) {
         const float q = fminf(p.wt, 1.0f);
-        if (!(b1.c < q)) { cnt_add(sm, FLR_C_RR_KILLS); finish(R, p); return c; }
+        if (!(b1.c < q)) { end = FLR_C_RR_KILLS; return c; }
         p.wt = p.wt < 1.0f ? 1.0f : p.wt;
     }
     if (!(isfinite(p.wt) && isfinite(p.x.x) && isfinite(p.x.y) && isfinite(p.x.z))) {
-        cnt_add(sm, FLR_C_NONFINITE);
-        finish(R, p);
+        end = FLR_C_NONFINITE;
         c.valid = false;
+    }
+    return c;
+}
+
+template <class M>
+__device__ __forceinline__ Conn track_step_hero(const M &m, const RunDev &R, const Smem &sm, Path &p,
+                                                HeroSet &h, RegCnt &rc)
+{
+    int end = -1;
+    const Conn c = track_body_hero(m, R, sm, p, h, rc, end);
+    if (end >= 0) {
+        cnt_add_any(sm, end);
+        finish(R, p);
     }
     return c;
 }
@@ -1884,7 +1958,7 @@ __global__ void __launch_bounds__(256) k_trace_wavefront(SceneDev S, RunDev R)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SmemLayout L = smem_layout(S.B, FLR_FORM_WAVEFRONT, blockDim.x);
-    const Smem sm = block_prologue(S, smem_raw, L, R.tallies);
+    const Smem sm = block_prologue(S, smem_raw, L, R.tallies, true);
     const int cap = 2 * blockDim.x;
     Queue q;
     {
@@ -1907,8 +1981,9 @@ __global__ void __launch_bounds__(256) k_trace_wavefront(SceneDev S, RunDev R)
     Path p;
     p.alive = false;
     bool exhausted = false;
-    const int regroup = R.regroup > 0 ? R.regroup : 8;
-    for (long long round = 0;; ++round) {
+    const int regroup = R.regroup > 0 ? min(R.regroup, MAX_REGROUP) : 8;
+    for (uint32_t round = 1;; ++round) {
+        if (round % CARRY_ROUNDS == 0u) counters_carry(sm);
         // stepping phase: at most `regroup` steps or one queued connection per thread
         for (int s = 0; s < regroup; ++s) {
             if (!p.alive) {
@@ -2391,7 +2466,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, (MODE == WM_RENDER && !MC) ? 5 : 4
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SmemLayout L = smem_layout(S.B, FLR_FORM_WAVEFRONT_WARP, blockDim.x);
-    const Smem sm = block_prologue(S, smem_raw, L, R.tallies);
+    const Smem sm = block_prologue(S, smem_raw, L, R.tallies, true);
     const MedS_<true, MC, IF, LZ> m{S, sm};
     constexpr unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2420,8 +2495,9 @@ __global__ void __launch_bounds__(WARP_BLOCK, (MODE == WM_RENDER && !MC) ? 5 : 4
     int ord = 0;                       // connections of the lane's path so far (adjoint passes)
     float tot = 0.0f, pre = 0.0f;      // pass 2: sum of the path's a_k, and of those seen so far
     float gsig = 0.0f;                 // pass 2: this lane's share of dL/dsigma_s
-    const int regroup = R.regroup > 0 ? R.regroup : 1;
-    while (true) {
+    const int regroup = R.regroup > 0 ? min(R.regroup, MAX_REGROUP) : 1;
+    for (uint32_t round = 1;; ++round) {
+        if (round % CARRY_ROUNDS == 0u) counters_carry(sm);
         // Tracking: at most `regroup` steps or one queued connection per lane. Lanes whose path
         // ended wait until SPAWN_MIN of them (or all) can start new paths together: the source
         // sampling then runs for several lanes at once instead of in most rounds for one or two
@@ -2831,7 +2907,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, 5) k_trace_pool(SceneDev S, RunDev
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SmemLayout L = smem_layout(S.B, FLR_FORM_WAVEFRONT_POOL, blockDim.x);
-    const Smem sm = block_prologue(S, smem_raw, L, R.tallies);
+    const Smem sm = block_prologue(S, smem_raw, L, R.tallies, true);
     const MedS_<true, false, IF> m{S, sm};
     constexpr unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2871,7 +2947,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, 5) k_trace_pool(SceneDev S, RunDev
     float gsig = 0.0f;
     const AdjDev A{};
     bool exhausted = false;
-    while (true) {
+    for (uint32_t round = 1;; ++round) {
+        if (round % CARRY_ROUNDS == 0u) counters_carry(sm);
         const int s0 = P.status[lane], s1 = P.status[lane + 32];
         const unsigned tlo = __ballot_sync(FULL, s0 == PS_TRACK), thi = __ballot_sync(FULL, s1 == PS_TRACK);
         const unsigned elo = __ballot_sync(FULL, s0 == PS_EVENT), ehi = __ballot_sync(FULL, s1 == PS_EVENT);
@@ -3021,7 +3098,7 @@ __host__ __device__ inline SmemLayout hero_warp_layout(int B, int block)
     L.tal_off_bytes = off;
     L.tal_global = true;
     L.cnt_off_bytes = off;
-    off += FLR_NCOUNTERS * 8;
+    off += FLR_NCOUNTERS * 12;
     off = ((off + 15) / 16) * 16;
     L.queue_off_bytes = off;
     off += (block / 32) * (HQ_CAP * HQ_WORDS * 4 + 8);
@@ -3180,7 +3257,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, 4) k_trace_hero_warp(SceneDev S, R
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SmemLayout L = hero_warp_layout(S.B, blockDim.x);
-    const Smem sm = block_prologue(S, smem_raw, L, R.tallies);
+    const Smem sm = block_prologue(S, smem_raw, L, R.tallies, true);
     const MedS_<true, false> m{S, sm};
     constexpr unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -3212,7 +3289,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, 4) k_trace_hero_warp(SceneDev S, R
     p.alive = false;
     HeroSet h;
     bool exhausted = false;
-    while (true) {
+    for (uint32_t round = 1;; ++round) {
+        if (round % CARRY_ROUNDS == 0u) counters_carry(sm);
         const bool spawn_now = __popc(__ballot_sync(FULL, !p.alive && !exhausted)) >= SPAWN_MIN ||
                                __ballot_sync(FULL, p.alive) == 0u;
         if (!p.alive) {
@@ -3586,7 +3664,7 @@ __global__ void __launch_bounds__(256, 2) k_trace_camera_warp(SceneDev S, RunDev
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SmemLayout L = smem_layout(S.B, FLR_FORM_PLAIN, blockDim.x);
-    const Smem sm = block_prologue(S, smem_raw, L, R.tallies);
+    const Smem sm = block_prologue(S, smem_raw, L, R.tallies, true);
     const MedS_<false> m{S, sm};
     constexpr unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -3601,7 +3679,8 @@ __global__ void __launch_bounds__(256, 2) k_trace_camera_warp(SceneDev S, RunDev
     CamPath cp;
     cp.alive = false;
     bool exhausted = false;
-    while (true) {
+    for (uint32_t round = 1;; ++round) {
+        if (round % CARRY_ROUNDS == 0u) counters_carry(sm);
         const bool spawn_now = __popc(__ballot_sync(FULL, !cp.alive && !exhausted)) >= SPAWN_MIN ||
                                __ballot_sync(FULL, cp.alive) == 0u;
         if (!cp.alive) {
@@ -3759,18 +3838,24 @@ __device__ __forceinline__ void counters_epilogue(const RunDev &R, const Smem &s
     __syncthreads();
     budget_flag(R, sm);
     for (int i = threadIdx.x; i < FLR_NCOUNTERS; i += blockDim.x)
-        if (sm.cnt[i]) atomicAdd(&R.counters[i], sm.cnt[i]);
+        if (cnt_total(sm, i)) atomicAdd(&R.counters[i], cnt_total(sm, i));
 }
 
-__global__ void __launch_bounds__(256) k_trace_batch(BatchDev Bt, RunDev R)
+__global__ void __launch_bounds__(256, 4) k_trace_batch(BatchDev Bt, RunDev R)
 {
     __shared__ unsigned long long s_cnt[FLR_NCOUNTERS];
-    for (int i = threadIdx.x; i < FLR_NCOUNTERS; i += blockDim.x) s_cnt[i] = 0ull;
+    __shared__ uint32_t s_cnt32[FLR_NCOUNTERS];
+    for (int i = threadIdx.x; i < FLR_NCOUNTERS; i += blockDim.x) {
+        s_cnt[i] = 0ull;
+        s_cnt32[i] = 0u;
+    }
     __syncthreads();
     Smem sm;
     sm.sig_a = sm.cdf = sm.maj = sm.inv_maj = sm.qy = nullptr;
     sm.tal = nullptr;
     sm.cnt = s_cnt;
+    sm.cnt32 = s_cnt32;
+    sm.persistent = true;
     RegCnt rc = {0, 0, 0, 0, 0, 0, 0};
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -3781,7 +3866,8 @@ __global__ void __launch_bounds__(256) k_trace_batch(BatchDev Bt, RunDev R)
     int cm = 0;                                        // warp's current chunk (warp-uniform)
     unsigned long long cnext = 0ull, cend = 0ull;
     bool done = false;
-    while (true) {
+    for (uint32_t round = 1;; ++round) {
+        if (round % CARRY_ROUNDS == 0u) counters_carry(sm);
         unsigned need = __ballot_sync(FULL, !p.alive);
         while (need != 0u && !done) {
             if (cnext >= cend) {
