@@ -999,12 +999,13 @@ __device__ __forceinline__ void finish(const RunDev &R, Path &p)
     if (R.path_events) R.path_events[p.pid - R.path_offset] = (uint32_t)p.n_events;
 }
 
-template <class M>
-__device__ __forceinline__ Conn spawn(const M &m, const RunDev &R, const Smem &sm, uint64_t pid,
-                                      Path &p, int *emitter = nullptr)
+// Starts path `pid` from the blocks of its spawn counter: s0 is slot 0, s1() gives slot 1 (drawn only
+// where it is needed).
+template <class M, class Block1>
+__device__ __forceinline__ Conn spawn_from(const M &m, const RunDev &R, const Smem &sm, uint64_t pid,
+                                           Path &p, int *emitter, const U4 &s0, const Block1 &block1)
 {
     cnt_add(sm, FLR_C_PATHS);
-    const U4 s0 = m.rng(R, pid, STEP_SPAWN, 0u);
     int k = 0;
     const int ne = m.n_emitters();
     while (k < ne - 1 && !(m.em_cdf(k) > s0.a)) ++k;
@@ -1024,7 +1025,7 @@ __device__ __forceinline__ Conn spawn(const M &m, const RunDev &R, const Smem &s
     Conn c;
     c.valid = false;
     if (e.kind == FLR_SOURCE_LAMBERTIAN) {
-        const U4 s1 = m.rng(R, pid, STEP_SPAWN, 1u);
+        const U4 s1 = block1();
         p.w = cosine_dir(s0.d, s1.a, e.axis, e.sign);
         if (m.sensor() && !R.paper_mode) {   // the paper's film holds fluorescence only
             c = Conn{p.x, p.wt, p.bin, 2 * e.axis + (e.sign > 0.0f ? 1 : 0), pid, STEP_SPAWN, true};
@@ -1035,7 +1036,7 @@ __device__ __forceinline__ Conn spawn(const M &m, const RunDev &R, const Smem &s
     if (m.iface() && e.entry >= 0) {
         // entering the solution through a dielectric face (coin: spawn slot 1, word 1): the
         // Fresnel-reflected share leaves through that face, the rest refracts inward by Snell
-        const U4 s1 = m.rng(R, pid, STEP_SPAWN, 1u);
+        const U4 s1 = block1();
         const int f = e.entry, k = f >> 1;
         const float wk = comp(p.w, k);
         float ct;
@@ -1053,6 +1054,14 @@ __device__ __forceinline__ Conn spawn(const M &m, const RunDev &R, const Smem &s
     }
     p.iw = inv_dir(p.w);
     return c;
+}
+
+template <class M>
+__device__ __forceinline__ Conn spawn(const M &m, const RunDev &R, const Smem &sm, uint64_t pid,
+                                      Path &p, int *emitter = nullptr)
+{
+    return spawn_from(m, R, sm, pid, p, emitter, m.rng(R, pid, STEP_SPAWN, 0u),
+                      [&] { return m.rng(R, pid, STEP_SPAWN, 1u); });
 }
 
 // Decisions that need no grid read. Where a medium has grids but no solvent mask (s(x) = 1), every
@@ -1080,8 +1089,8 @@ struct NoObs {
 // One tracking step (null or real collision, wall bounce or escape). Returns the connection the
 // step asks for, if any; a step that ends the path says which counter it ends on in `end`.
 template <class M, class Obs>
-__device__ __forceinline__ Conn track_body(const M &m, const RunDev &R, const Smem &sm, Path &p,
-                                           RegCnt &rc, const Obs &obs, int &end)
+__device__ __forceinline__ Conn track_body(const M &m, const RunDev &R, const Smem &sm, Path &p, const U4 &b0,
+                                           const U4 &b1, RegCnt &rc, const Obs &obs, int &end)
 {
     Conn c;
     c.valid = false;
@@ -1090,10 +1099,6 @@ __device__ __forceinline__ Conn track_body(const M &m, const RunDev &R, const Sm
         return c;
     }
     rc.steps++;
-    const U4 b0 = m.rng(R, p.pid, p.step, 0u);
-    // The second block serves real events and wall bounces only, but some lane of a warp nearly
-    // always needs it: drawing it here, beside the first, overlaps the two Philox chains.
-    const U4 b1 = m.rng(R, p.pid, p.step, 1u);
     int face;
     const float te = exit_distance(m, p.x, p.w, p.iw, face);
     float sb, tf;
@@ -1306,12 +1311,81 @@ __device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Sm
                                            RegCnt &rc, const Obs &obs = Obs())
 {
     int end = -1;
-    const Conn c = track_body(m, R, sm, p, rc, obs, end);
+    const U4 b0 = m.rng(R, p.pid, p.step, 0u);
+    // The second block serves real events and wall bounces only, but some lane of a warp nearly
+    // always needs it: drawing it here, beside the first, overlaps the two Philox chains.
+    const U4 b1 = m.rng(R, p.pid, p.step, 1u);
+    const Conn c = track_body(m, R, sm, p, b0, b1, rc, obs, end);
     if (end >= 0) {
         cnt_add_any(sm, end);
         finish(R, p);
     }
     return c;
+}
+
+// The rounds of the persistent forms: a lane whose path ended takes the next path id with
+// path_claimed() and makes its spawn in the next round's step, which draws the blocks of whatever
+// counter the path stands at (STEP_SPAWN for a claimed one). So the Philox rounds of a spawn run for
+// the tracking lanes and the spawning ones at once, and no lane waits for others to start with it.
+__device__ __forceinline__ void path_claimed(Path &p, uint64_t pid)
+{
+    p.pid = pid;
+    p.step = STEP_SPAWN;
+    p.alive = true;
+}
+
+template <class M, class Obs = NoObs>
+__device__ __forceinline__ Conn spawn_or_track(const M &m, const RunDev &R, const Smem &sm, Path &p, RegCnt &rc,
+                                               const Obs &obs = Obs())
+{
+    int end = -1;
+    const U4 b0 = m.rng(R, p.pid, p.step, 0u), b1 = m.rng(R, p.pid, p.step, 1u);
+    if (p.step == STEP_SPAWN) return spawn_from(m, R, sm, p.pid, p, nullptr, b0, [&] { return b1; });
+    const Conn c = track_body(m, R, sm, p, b0, b1, rc, obs, end);
+    if (end >= 0) {
+        cnt_add_any(sm, end);
+        finish(R, p);
+    }
+    return c;
+}
+
+// Path ids of one warp, in shared memory: taken from the launch's counter some at a time (few enough that a
+// small launch spreads over all warps, 32 beyond), handed to the lanes that ask, in order. claim_path()
+// gives a lane its id; a warp whose ids run out in a round serves the rest of its lanes in the next one.
+struct PathIds {
+    unsigned long long next;
+    int left;
+    int dry;   // the launch has no more ids
+};
+
+__device__ __forceinline__ bool ids_left(const PathIds *ids) { return ids->left > 0 || !ids->dry; }
+
+// Called by the whole warp; need: the lanes that ask. True if the lane got path R.path_offset + i.
+__device__ __forceinline__ bool claim_path(PathIds *ids, const RunDev &R, unsigned need, unsigned long long &i)
+{
+    const int lane = threadIdx.x & 31;
+    if (ids->left == 0) {
+        __syncwarp();
+        if (lane == 0) {
+            const unsigned long long warps = gridDim.x * (blockDim.x >> 5), n = R.n_paths;
+            const unsigned long long chunk = min(max(n / warps, 1ull), 32ull);
+            const unsigned long long first = atomicAdd(R.work_counter, chunk);
+            ids->next = first;
+            ids->dry = first + chunk >= n;
+            ids->left = first < n ? (int)min(chunk, n - first) : 0;
+        }
+        __syncwarp();
+    }
+    const int rank = __popc(need & ((1u << lane) - 1u)), left = ids->left;
+    i = ids->next + (unsigned long long)rank;
+    __syncwarp();
+    if (lane == 0) {
+        const int taken = min(__popc(need), left);
+        ids->next += (unsigned long long)taken;
+        ids->left = left - taken;
+    }
+    __syncwarp();
+    return ((need >> lane) & 1u) && rank < left;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1322,20 +1396,23 @@ struct SmemLayout {
 };
 
 // Per-warp connection queue of the warp-regrouped form: capacity and drain threshold. A drain starts
-// once WQ_DRAIN records wait; one tracking round adds at most 32, so the queue never wraps. Longer
-// queues drain less often and amortise each drain's tail (measured on the Cornell box: 128 -> 256 ->
-// 320 records gave 26.0 -> 24.0 -> 23.6 ms per step, with the drains of that time); five blocks of
-// 128 threads (WARP_BLOCK, at most 102 registers) per SM measured 3 % faster than two blocks of 256
-// with 416-record queues. With drains that claim every iteration the optimum moved down: 256
-// records (drained at 224) gave 12.93 ms, against 13.14 (320 / 288), 12.97 (224 / 192), 13.2
-// (192 / 160) and 13.45 ms (160 / 128); the block count stays five (registers), and the shared
-// memory no longer held by queues is left to the L1. The adjoint's and the local-majorant
-// instances keep four blocks (128 registers): with five they spill.
+// once WQ_DRAIN records wait; one tracking round adds at most 32, so the queue never wraps. A drain begins
+// its records 32 together and keeps its unfinished marches (wq_drain), so it has no tail to spread over a longer
+// queue: 128 records measured as 224 (the light sheet 171.2 and 171 ms, the Cornell box 10.5 and 10.6).
+// Four blocks of 128 threads (at most 128 registers) share an SM: with five (96 registers) the two kinds of
+// work of a drain spill in their loops, and every workload took 20 to 60 % longer.
 constexpr int WARP_BLOCK = 128;   // threads per block of the warp-regrouped form
-constexpr int WQ_CAP = 256;
-constexpr int WQ_DRAIN = 224;
-constexpr int SPAWN_MIN = 8;   // lanes that start new paths together
+constexpr int WARP_BLOCKS = 4;    // blocks per SM its registers are bounded for
+constexpr int WQ_CAP = 128;
+constexpr int WQ_DRAIN = WQ_CAP - 32;
+constexpr int MS_CAP = 64;        // stack of marches that wait: fewer than 32 before 32 records are begun
+constexpr int MS_WORDS = 19;      // 4-byte fields per waiting march
+constexpr int DRAIN_KEEP = 16;    // a drain ends once fewer lanes would go on (8 and 24 measured the same)
+constexpr int SPAWN_MIN = 8;      // lanes that start new paths together (hero, camera; pass 2 of the adjoint)
+constexpr int CLAIM_MIN = 4;      // lanes that take path ids together (the light sheet: 1: 180, 4: 182, 8: 189 ms)
+constexpr int WARP_WORDS = 6;     // head, tail and PathIds of a warp (8-byte aligned)
 static_assert(WQ_DRAIN + 31 < WQ_CAP, "warp queue overflow");
+static_assert(MS_CAP >= 64 && DRAIN_KEEP <= 32, "march stack overflow");
 
 // Path-pool form (k_trace_pool): slots per warp, connection queue, per-warp shared memory.
 constexpr int POOL_SLOTS = 64;   // lane l keeps the states of slots l and l + 32
@@ -1364,7 +1441,7 @@ __host__ __device__ inline SmemLayout smem_layout(int B, int form, int block)
     off = ((off + 15) / 16) * 16;
     L.queue_off_bytes = off;
     if (form == FLR_FORM_WAVEFRONT) off += 2 * block * 32 + 16;
-    if (form == FLR_FORM_WAVEFRONT_WARP) off += (block / 32) * (WQ_CAP * 32 + 8);
+    if (form == FLR_FORM_WAVEFRONT_WARP) off += (block / 32) * (WQ_CAP * 32 + MS_CAP * MS_WORDS * 4 + WARP_WORDS * 4);
     if (form == FLR_FORM_WAVEFRONT_POOL) off += (block / 32) * POOL_WARP_BYTES;
     L.total_bytes = off;
     return L;
@@ -1684,8 +1761,8 @@ __device__ __forceinline__ void hero_tally(const M &m, int row, const HeroSet &h
 // One tracking step of a hero path: the single-wavelength step (track_step) with the set's
 // majorant, the weights re-balanced at null collisions and the tallies split among the members.
 template <class M>
-__device__ __forceinline__ Conn track_body_hero(const M &m, const RunDev &R, const Smem &sm, Path &p,
-                                                HeroSet &h, RegCnt &rc, int &end)
+__device__ __forceinline__ Conn track_body_hero(const M &m, const RunDev &R, const Smem &sm, Path &p, const U4 &b0,
+                                                const U4 &b1, HeroSet &h, RegCnt &rc, int &end)
 {
     Conn c;
     c.valid = false;
@@ -1694,8 +1771,6 @@ __device__ __forceinline__ Conn track_body_hero(const M &m, const RunDev &R, con
         return c;
     }
     rc.steps++;
-    const U4 b0 = m.rng(R, p.pid, p.step, 0u);
-    const U4 b1 = m.rng(R, p.pid, p.step, 1u);
     int face;
     const float te = exit_distance(m, p.x, p.w, p.iw, face);
     const float sb = h.sb;
@@ -1865,7 +1940,8 @@ __device__ __forceinline__ Conn track_step_hero(const M &m, const RunDev &R, con
                                                 HeroSet &h, RegCnt &rc)
 {
     int end = -1;
-    const Conn c = track_body_hero(m, R, sm, p, h, rc, end);
+    const U4 b0 = m.rng(R, p.pid, p.step, 0u), b1 = m.rng(R, p.pid, p.step, 1u);
+    const Conn c = track_body_hero(m, R, sm, p, b0, b1, h, rc, end);
     if (end >= 0) {
         cnt_add_any(sm, end);
         finish(R, p);
@@ -2289,10 +2365,11 @@ __global__ void __launch_bounds__(256) k_frozen_sums(SceneDev S, RunDev R, PertD
 // ---------------------------------------------------------------------------------------------
 // Wavefront form with per-warp regrouping and pull-based connection drains. Each warp queues its
 // lanes' sensor connections in shared memory (up to WQ_CAP records). Once WQ_DRAIN records are
-// waiting (or the work is done) the warp drains the queue: every lane advances its own
-// ratio-tracking march by one step per iteration and claims the next record as soon as its march
-// ends, so the lanes stay busy until the queue runs dry instead of waiting for the longest march
-// of a fixed batch. The marches consume their random numbers exactly as transmittance() does, so
+// waiting (or the work is done) the warp drains the queue (wq_drain): records are begun 32 together,
+// then every lane advances its own ratio-tracking march by one step per iteration and takes the next one
+// as soon as its march ends. Against claims of single records in every iteration, and spawns of eight
+// lanes apart from the tracking step: the light sheet 186.7 -> 171.2 ms, the Cornell box 11.5 -> 10.5 ms (a
+// preview of 97 x 71 pixels 1.14 -> 0.92), a fit step 17.5 -> 17.2 ms. The marches consume their random numbers exactly as transmittance() does, so
 // every launch form gives the same film up to the order of the fp32 film atomics.
 //
 // The same kernel runs the two passes of the adjoint replay (MODE):
@@ -2313,23 +2390,24 @@ struct March {
     float tl, t, T, isb, wg;   // wg: intensity x importance (render, pass 1) or a_k (pass 2)
     int b, pix, it, ord;
     uint64_t pid;
+    float u2;                  // the roulette coin of the waiting point, where it is already drawn
     MarchRng g;                // the connection's uniform stream
 };
 
 // A queued connection record: position, weight (pass 2: a_k), bin, vertex kind, ordinal along
 // its path, RNG coordinates. bin < 256 (FLR_MAX_BINS), vertex kind + 1 in 0..6.
-__device__ __forceinline__ void wq_push(const Queue &q, const Conn &c, float w, int ord)
+__device__ __forceinline__ void wq_push(const Queue &q, const Path &p, float w, int lamb, int ord)
 {
-    const int slot = atomicAdd(&q.head_tail[1], 1) % WQ_CAP;
-    (void)FLR_CHK(q.head_tail[1] <= WQ_CAP, CK_QUEUE, slot);   // a wrap would overwrite a waiting record
-    q.x[slot] = c.x.x;
-    q.y[slot] = c.x.y;
-    q.z[slot] = c.x.z;
+    const int slot = atomicAdd(&q.head_tail[1], 1);
+    if (!FLR_CHK(slot < WQ_CAP, CK_QUEUE, slot)) return;
+    q.x[slot] = p.x.x;
+    q.y[slot] = p.x.y;
+    q.z[slot] = p.x.z;
     q.w[slot] = w;
-    q.bin_lamb[slot] = (c.bin & 0xFF) | ((c.lamb + 1) << 8) | (min(ord, WQ_ORD_MAX) << 11);
-    q.pid_lo[slot] = (uint32_t)c.pid;
-    q.pid_hi[slot] = (uint32_t)(c.pid >> 32);
-    q.step[slot] = c.step;
+    q.bin_lamb[slot] = (p.bin & 0xFF) | ((lamb + 1) << 8) | (min(ord, WQ_ORD_MAX) << 11);
+    q.pid_lo[slot] = (uint32_t)p.pid;
+    q.pid_hi[slot] = (uint32_t)(p.pid >> 32);
+    q.step[slot] = p.step - 1u;   // the step just made; STEP_SPAWN after a spawn
 }
 
 // The end of a march that reached the sensor side of the box.
@@ -2408,10 +2486,13 @@ __device__ __forceinline__ bool march_begin(const SceneDev &S, const RunDev &R, 
 
 __device__ __forceinline__ float march_uniform(const RunDev &, March &mc) { return march_next(mc.g); }
 
-// One ratio-tracking step (the body of transmittance()'s loop); returns false when the march ends.
-template <int MODE, bool LZ = false>
-__device__ __forceinline__ bool march_step(const SceneDev &S, const RunDev &R, const Smem &sm,
-                                           const AdjDev &A, March &mc, RegCnt &rc, float &gsig)
+// One ratio-tracking step (the body of transmittance()'s loop) in two halves. march_advance draws the
+// next point of the march; false when there is none: the march reached the sensor side (its value is
+// deposited) or its roulette coin ends it whatever the matter there is. march_matter reads the matter
+// at that point and updates the estimate; false when the roulette ends the march.
+template <int MODE, bool LZ>
+__device__ __forceinline__ bool march_advance(const SceneDev &S, const RunDev &R, const Smem &sm,
+                                              const AdjDev &A, March &mc, RegCnt &rc)
 {
     if (mc.it >= MAX_CONNECT_STEPS) {
         cnt_add(sm, FLR_C_CONNECT_BUDGET);
@@ -2425,17 +2506,24 @@ __device__ __forceinline__ bool march_step(const SceneDev &S, const RunDev &R, c
         return false;
     }
     rc.connect_steps++;
-    const MedS m{S, sm};
-    float u2 = -1.0f;   // the roulette coin, when the bound below draws it first
+    mc.u2 = -1.0f;
     if (MODE == WM_RENDER && LZ && !S.homogeneous && S.solvent == nullptr) {
         // upper bound of the updated estimate (minorant_known): a coin that fails against it ends
         // the march whatever sigma_t is here
         const float tu = mc.T * fmaxf(0.0f, 1.0f - (S.sigma_s + S.sigma_a0) * mc.isb);
         if (tu < RT_RR_THRESHOLD) {
-            u2 = march_uniform(R, mc);
-            if (!(u2 * RT_RR_THRESHOLD < tu)) return false;
+            mc.u2 = march_uniform(R, mc);
+            if (!(mc.u2 * RT_RR_THRESHOLD < tu)) return false;
         }
     }
+    return true;
+}
+
+template <int MODE, bool LZ>
+__device__ __forceinline__ bool march_matter(const SceneDev &S, const RunDev &R, const Smem &sm,
+                                             const AdjDev &A, March &mc, RegCnt &rc, float &gsig)
+{
+    const MedS m{S, sm};
     const float3 p = make_float3(mc.x.x + mc.t * mc.dir.x, mc.x.y + mc.t * mc.dir.y,
                                  mc.x.z + mc.t * mc.dir.z);
     const int4 ec = S.sk > 0 ? empty_cell(m, p) : make_int4(0, 0, 0, 0);
@@ -2451,7 +2539,7 @@ __device__ __forceinline__ bool march_step(const SceneDev &S, const RunDev &R, c
     }
     constexpr bool ADJ = MODE != WM_RENDER;
     if (mc.T < (ADJ ? RT_RR_ADJ_THRESHOLD : RT_RR_THRESHOLD)) {
-        if (u2 < 0.0f) u2 = march_uniform(R, mc);
+        const float u2 = LZ && mc.u2 >= 0.0f ? mc.u2 : march_uniform(R, mc);
         if (ADJ ? u2 < 0.5f : u2 * RT_RR_THRESHOLD < mc.T) {
             mc.T = ADJ ? 2.0f * mc.T : RT_RR_THRESHOLD;
         } else {
@@ -2461,8 +2549,134 @@ __device__ __forceinline__ bool march_step(const SceneDev &S, const RunDev &R, c
     return true;
 }
 
+// The whole step, for the path-pool form's drains.
+template <int MODE>
+__device__ __forceinline__ bool march_step(const SceneDev &S, const RunDev &R, const Smem &sm,
+                                           const AdjDev &A, March &mc, RegCnt &rc, float &gsig)
+{
+    return march_advance<MODE, false>(S, R, sm, A, mc, rc) && march_matter<MODE, false>(S, R, sm, A, mc, rc, gsig);
+}
+
+// A march that waits at its next point, one word of each field per slot of the warp's stack.
+template <int MODE, bool LZ>
+__device__ __forceinline__ void stack_store(float *st, int slot, const March &mc)
+{
+    if (!FLR_CHK(slot < MS_CAP, CK_QUEUE, slot)) return;
+    float *f = st + slot;
+    f[0 * MS_CAP] = mc.x.x;
+    f[1 * MS_CAP] = mc.x.y;
+    f[2 * MS_CAP] = mc.x.z;
+    f[3 * MS_CAP] = mc.dir.x;
+    f[4 * MS_CAP] = mc.dir.y;
+    f[5 * MS_CAP] = mc.dir.z;
+    f[6 * MS_CAP] = mc.tl;
+    f[7 * MS_CAP] = mc.t;
+    f[8 * MS_CAP] = mc.T;
+    f[9 * MS_CAP] = mc.wg;
+    f[10 * MS_CAP] = __int_as_float(mc.pix);
+    f[11 * MS_CAP] = __int_as_float(mc.b | (mc.it << 8));
+    f[12 * MS_CAP] = __uint_as_float(mc.g.s0);
+    f[13 * MS_CAP] = __uint_as_float(mc.g.s1);
+    f[14 * MS_CAP] = __uint_as_float(mc.g.s2);
+    f[15 * MS_CAP] = __uint_as_float(mc.g.s3);
+    if (LZ) f[16 * MS_CAP] = mc.u2;
+    if (MODE == WM_ADJ_WEIGHTS) {
+        f[16 * MS_CAP] = __int_as_float(mc.ord);
+        f[17 * MS_CAP] = __uint_as_float((uint32_t)mc.pid);
+        f[18 * MS_CAP] = __uint_as_float((uint32_t)(mc.pid >> 32));
+    }
+}
+
+template <int MODE, bool LZ>
+__device__ __forceinline__ void stack_load(const Smem &sm, const float *st, int slot, March &mc)
+{
+    const float *f = st + slot;
+    mc.x = make_float3(f[0 * MS_CAP], f[1 * MS_CAP], f[2 * MS_CAP]);
+    mc.dir = make_float3(f[3 * MS_CAP], f[4 * MS_CAP], f[5 * MS_CAP]);
+    mc.idir = inv_dir(mc.dir);
+    mc.tl = f[6 * MS_CAP];
+    mc.t = f[7 * MS_CAP];
+    mc.T = f[8 * MS_CAP];
+    mc.wg = f[9 * MS_CAP];
+    mc.pix = __float_as_int(f[10 * MS_CAP]);
+    const int bi = __float_as_int(f[11 * MS_CAP]);
+    mc.b = bi & 0xFF;
+    mc.it = bi >> 8;
+    mc.isb = sm.inv_maj[mc.b];
+    mc.g = MarchRng{__float_as_uint(f[12 * MS_CAP]), __float_as_uint(f[13 * MS_CAP]),
+                    __float_as_uint(f[14 * MS_CAP]), __float_as_uint(f[15 * MS_CAP])};
+    mc.u2 = LZ ? f[16 * MS_CAP] : -1.0f;
+    if (MODE == WM_ADJ_WEIGHTS) {
+        mc.ord = __float_as_int(f[16 * MS_CAP]);
+        mc.pid = ((uint64_t)__float_as_uint(f[18 * MS_CAP]) << 32) | __float_as_uint(f[17 * MS_CAP]);
+    }
+}
+
+// Makes the `avail` queued connections of the warp (and goes on with the marches an earlier drain left
+// on the stack). Whenever the stack cannot serve every idle lane, 32 records are begun together: their
+// geometry, their Philox block and their first tentative point, which already ends most connections of
+// a dense medium. What is left goes to the stack without gaps, and lanes whose march ends take
+// the next one from it, so both kinds of work run on full warps. A drain that runs out of records puts
+// its last marches back on the stack (fewer than DRAIN_KEEP lanes would go on) unless it is the last.
+template <int MODE, bool MC, bool LZ>
+__device__ __forceinline__ void wq_drain(const SceneDev &S, const RunDev &R, const Smem &sm, const AdjDev &A,
+                                         const Queue &q, float *stack, int avail, bool last, RegCnt &rc, float &gsig)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned lower = (1u << lane) - 1u;
+    int depth = q.head_tail[0];
+    const int least = last ? 1 : 32;   // only the last drain begins fewer than 32 records together
+    March mc;
+    bool active = false;
+    for (;;) {
+        const unsigned idle = __ballot_sync(FULL, !active);
+        const int n_idle = __popc(idle);
+        while (depth < n_idle && avail >= least) {
+            March nw;
+            bool go = false;
+            const int k = avail - 1 - lane;
+            if (k >= 0) {
+                const int bl = q.bin_lamb[k];
+                const uint64_t pid = ((uint64_t)q.pid_hi[k] << 32) | q.pid_lo[k];
+                go = march_begin<MODE, MC>(S, R, sm, A, make_float3(q.x[k], q.y[k], q.z[k]), bl & 0xFF, q.w[k],
+                                           ((bl >> 8) & 7) - 1,
+                                           MODE == WM_ADJ_WEIGHTS ? (int)((unsigned)bl >> 11) : 0, pid, q.step[k],
+                                           nw, rc, gsig) &&
+                     march_advance<MODE, LZ>(S, R, sm, A, nw, rc);
+            }
+            avail = max(avail - 32, 0);
+            const unsigned going = __ballot_sync(FULL, go);
+            if (go) stack_store<MODE, LZ>(stack, depth + __popc(going & lower), nw);
+            depth += __popc(going);
+            __syncwarp();
+        }
+        const int rank = __popc(idle & lower);
+        if (!active && rank < depth) {
+            stack_load<MODE, LZ>(sm, stack, depth - 1 - rank, mc);
+            active = true;
+        }
+        depth = max(depth - n_idle, 0);
+        const unsigned act = __ballot_sync(FULL, active);
+        if (act == 0u) break;
+        if (avail < least && depth == 0 && !last && __popc(act) < DRAIN_KEEP) {
+            if (active) stack_store<MODE, LZ>(stack, __popc(act & lower), mc);
+            depth = __popc(act);
+            break;
+        }
+        if (active) active = march_matter<MODE, LZ>(S, R, sm, A, mc, rc, gsig) &&
+                             march_advance<MODE, LZ>(S, R, sm, A, mc, rc);
+    }
+    __syncwarp();
+    if (lane == 0) {
+        q.head_tail[0] = depth;
+        q.head_tail[1] = avail;
+    }
+    __syncwarp();
+}
+
 template <int MODE, bool MC, bool IF = true, bool LZ = false>
-__global__ void __launch_bounds__(WARP_BLOCK, (MODE == WM_RENDER && !MC) ? 5 : 4) k_trace_wavefront_warp(SceneDev S, RunDev R, AdjDev A)
+__global__ void __launch_bounds__(WARP_BLOCK, WARP_BLOCKS) k_trace_wavefront_warp(SceneDev S, RunDev R, AdjDev A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SmemLayout L = smem_layout(S.B, FLR_FORM_WAVEFRONT_WARP, blockDim.x);
@@ -2471,8 +2685,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, (MODE == WM_RENDER && !MC) ? 5 : 4
     constexpr unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nwarps = blockDim.x >> 5;
-    const unsigned lower = (1u << lane) - 1u;
     Queue q;
+    float *stack;
     {
         unsigned char *base = smem_raw + L.queue_off_bytes;
         float *f = reinterpret_cast<float *>(base) + warp * WQ_CAP * 8;
@@ -2484,114 +2698,72 @@ __global__ void __launch_bounds__(WARP_BLOCK, (MODE == WM_RENDER && !MC) ? 5 : 4
         q.pid_lo = reinterpret_cast<uint32_t *>(q.bin_lamb + WQ_CAP);
         q.pid_hi = q.pid_lo + WQ_CAP;
         q.step = q.pid_hi + WQ_CAP;
-        q.head_tail = reinterpret_cast<int *>(base + (size_t)nwarps * WQ_CAP * 32) + 2 * warp;
-        if (lane == 0) { q.head_tail[0] = 0; q.head_tail[1] = 0; }
+        stack = reinterpret_cast<float *>(base + (size_t)nwarps * WQ_CAP * 32) + warp * MS_CAP * MS_WORDS;
+        q.head_tail = reinterpret_cast<int *>(base + (size_t)nwarps * (WQ_CAP * 32 + MS_CAP * MS_WORDS * 4)) + WARP_WORDS * warp;
+        if (lane < WARP_WORDS) q.head_tail[lane] = 0;
     }
     __syncwarp();
     RegCnt rc = {0, 0, 0, 0, 0, 0, 0};
     Path p;
     p.alive = false;
-    bool exhausted = false;
+    PathIds *const ids = reinterpret_cast<PathIds *>(q.head_tail + 2);
     int ord = 0;                       // connections of the lane's path so far (adjoint passes)
     float tot = 0.0f, pre = 0.0f;      // pass 2: sum of the path's a_k, and of those seen so far
     float gsig = 0.0f;                 // pass 2: this lane's share of dL/dsigma_s
     const int regroup = R.regroup > 0 ? min(R.regroup, MAX_REGROUP) : 1;
     for (uint32_t round = 1;; ++round) {
         if (round % CARRY_ROUNDS == 0u) counters_carry(sm);
-        // Tracking: at most `regroup` steps or one queued connection per lane. Lanes whose path
-        // ended wait until SPAWN_MIN of them (or all) can start new paths together: the source
-        // sampling then runs for several lanes at once instead of in most rounds for one or two
-        // (measured: 21.5 -> 19.5 ms per Cornell-box step with 8).
-        const bool spawn_now = __popc(__ballot_sync(FULL, !p.alive && !exhausted)) >= SPAWN_MIN ||
-                               __ballot_sync(FULL, p.alive) == 0u;
-        for (int s = 0; s < regroup; ++s) {
-            if (MODE != WM_ADJ_GRAD) {
-                if (!p.alive) {
-                    if (exhausted || !spawn_now) break;
-                    const unsigned long long i = atomicAdd(R.work_counter, 1ull);
-                    if (i >= R.n_paths) { exhausted = true; break; }
-                    const Conn c = spawn(m, R, sm, R.path_offset + i, p);
-                    ord = 0;
-                    if (c.valid) {
-                        wq_push(q, c, c.w, ord);
-                        if (MODE == WM_ADJ_WEIGHTS) ++ord;
-                        break;
+        // Lanes whose path ended take the next path ids. Pass 2 reads a path's contributions there,
+        // so it waits until SPAWN_MIN lanes (or all) can read together.
+        const unsigned need = __ballot_sync(FULL, !p.alive);
+        if (need != 0u && ids_left(ids) &&
+            (__popc(need) >= (MODE == WM_ADJ_GRAD ? SPAWN_MIN : CLAIM_MIN) || need == FULL)) {
+            unsigned long long i;
+            if (claim_path(ids, R, need, i)) {
+                path_claimed(p, R.path_offset + i);
+                ord = 0;
+                if (MODE == WM_ADJ_GRAD) {
+                    // the path's contributions from pass 1, summed in path order
+                    const float *ak = A.ak + i * A.K;
+                    const float ov = A.ovf[i];
+                    bool nz = ov != 0.0f;
+                    tot = 0.0f;
+                    for (int k = 0; k < A.K; ++k) {
+                        const float a = ak[k];
+                        tot += a;
+                        nz |= a != 0.0f;
                     }
-                    continue;
+                    tot += ov;
+                    pre = 0.0f;
+                    p.alive = nz;   // otherwise there is nothing to differentiate
                 }
-                const Conn c = track_step(m, R, sm, p, rc);
+            }
+        }
+        // Tracking: at most `regroup` steps or one queued connection per lane.
+        for (int s = 0; s < regroup && p.alive; ++s) {
+            if (MODE != WM_ADJ_GRAD) {
+                const Conn c = spawn_or_track(m, R, sm, p, rc);
                 if (c.valid) {
-                    wq_push(q, c, c.w, MODE == WM_ADJ_WEIGHTS ? ord : 0);
+                    wq_push(q, p, c.w, c.lamb, MODE == WM_ADJ_WEIGHTS ? ord : 0);
                     if (MODE == WM_ADJ_WEIGHTS) ++ord;
                     break;
                 }
                 continue;
             }
             // pass 2 of the adjoint
-            Conn c;
-            if (!p.alive) {
-                if (exhausted || !spawn_now) break;
-                const unsigned long long i = atomicAdd(R.work_counter, 1ull);
-                if (i >= R.n_paths) { exhausted = true; break; }
-                c = spawn(m, R, sm, R.path_offset + i, p);
-                ord = 0;
-                // the path's contributions from pass 1, summed in path order
-                const float *ak = A.ak + i * A.K;
-                const float ov = A.ovf[i];
-                bool nz = ov != 0.0f;
-                tot = 0.0f;
-                for (int k = 0; k < A.K; ++k) {
-                    const float a = ak[k];
-                    tot += a;
-                    nz |= a != 0.0f;
-                }
-                tot += ov;
-                pre = 0.0f;
-                if (!nz) { p.alive = false; continue; }   // nothing to differentiate
-            } else {
-                c = track_step(m, R, sm, p, rc, AdjObs{S, sm, A, tot - pre, &gsig});
-            }
+            const Conn c = spawn_or_track(m, R, sm, p, rc, AdjObs{S, sm, A, tot - pre, &gsig});
             if (!c.valid) continue;
             const float a = ord < A.K ? __ldg(&A.ak[(p.pid - R.path_offset) * A.K + ord])
                                       : adjoint_weight<MC>(S, R, sm, A, c, rc);
             ++ord;
             pre += a;
-            if (a != 0.0f) { wq_push(q, c, a, 0); break; }
+            if (a != 0.0f) { wq_push(q, p, a, c.lamb, 0); break; }
         }
         __syncwarp();
-        const bool any = __any_sync(FULL, p.alive || !exhausted);
+        const bool any = __any_sync(FULL, p.alive) || ids_left(ids);
         const int avail = q.head_tail[1];
-        if (avail >= WQ_DRAIN || (!any && avail > 0)) {
-            // pull-based drain of all `avail` records; a lane whose march ended claims the next
-            // record in the next iteration (measured with the march streams: 13.14 ms per
-            // Cornell-box step and 33.3 ms per 8.4M light-sheet paths, against 13.28 / 35.5 ms
-            // claiming every second iteration, 13.70 / 36.3 every third and 14.20 / 37.1 every
-            // fourth; every second had been fastest while marches drew Philox blocks by phase)
-            March mc;
-            bool active = false;
-            int claimed = 0;
-            for (;;) {
-                const unsigned need = __ballot_sync(FULL, !active);
-                if (need != 0u && !active) {
-                    const int k = claimed + __popc(need & lower);
-                    if (k < avail) {
-                        const int bl = q.bin_lamb[k];
-                        const uint64_t pid = ((uint64_t)q.pid_hi[k] << 32) | q.pid_lo[k];
-                        active = march_begin<MODE, MC>(S, R, sm, A, make_float3(q.x[k], q.y[k], q.z[k]),
-                                                   bl & 0xFF, q.w[k], ((bl >> 8) & 7) - 1,
-                                                   MODE == WM_ADJ_WEIGHTS ? (int)((unsigned)bl >> 11) : 0,
-                                                   pid, q.step[k], mc, rc,
-                                                   gsig);
-                    }
-                }
-                claimed += __popc(need);
-                if (active) active = march_step<MODE, LZ>(S, R, sm, A, mc, rc, gsig);
-                if (!__any_sync(FULL, active) && claimed >= avail) break;
-            }
-            __syncwarp();
-            if (lane == 0) q.head_tail[1] = 0;
-            __syncwarp();
-        }
+        if (avail >= WQ_DRAIN || (!any && avail + q.head_tail[0] > 0))
+            wq_drain<MODE, MC, LZ>(S, R, sm, A, q, stack, avail, !any, rc, gsig);
         if (!any) break;
     }
     if (MODE == WM_RENDER) {
@@ -3887,8 +4059,7 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(BatchDev Bt, RunDev R)
             const int rank = __popc(need & lower);
             if (((need >> lane) & 1u) && (unsigned long long)rank < avail) {
                 mi = cm;
-                const MedB m{Bt.media + cm, Bt.B};
-                spawn(m, R, sm, cnext + (unsigned long long)rank, p);
+                path_claimed(p, cnext + (unsigned long long)rank);
             }
             const unsigned long long n_need = (unsigned long long)__popc(need);
             cnext += n_need < avail ? n_need : avail;
@@ -3897,7 +4068,7 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(BatchDev Bt, RunDev R)
         if (__ballot_sync(FULL, p.alive) == 0u && done) break;
         if (p.alive) {
             const MedB m{Bt.media + mi, Bt.B};
-            track_step(m, R, sm, p, rc);
+            spawn_or_track(m, R, sm, p, rc);
         }
     }
     counters_epilogue(R, sm, rc);

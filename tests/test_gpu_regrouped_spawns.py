@@ -1,0 +1,119 @@
+"""The persistent forms hand path ids to lanes from per-warp stocks, start their paths in the tracking step,
+begin connections 32 together and put unfinished marches aside. None of it may change a result: at path counts
+around the sizes of a warp, a stock and a launch, every form gives the plain form's counters, tallies and film
+bit for bit (both are exact sums). A batch of media is compared with the media one by one."""
+import numpy as np
+import pytest
+import torch
+
+import scenegen as sg
+from tests.gpu_common import require_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _cube(n):
+    return sg.cfg1_homogeneous_cube(n_paths=n, film=17)
+
+
+def _clear_cube(n):   # no extinction at all: every path crosses the box, nothing connects
+    sc = _cube(n)
+    sc["medium"] = sg.homogeneous_medium(1, conc=0.0, sigma_s=0.0)
+    return sc
+
+
+def _walled_cube(n):
+    sc = _cube(n)
+    sc["medium"] = sg.homogeneous_medium(1, conc=0.5, sigma_s=5.0, sigma_a0=0.3, wall_mask=0b011111, wall_albedo=0.9)
+    return sc
+
+
+def _cornell(n):
+    return sg.cfg2_cornell_box(width=19, height=23, grid=21, n_paths=n)
+
+
+def _sheet(n):
+    return sg.cfg5_light_sheet(grid=19, width=24, height=24, n_blobs=20, n_paths=n, albedo=0.999)
+
+
+def _vial(n):
+    return sg.vial_scene(width=20, height=20, n_paths=n)
+
+
+SCENES = {"cube": (_cube, [{}]), "clear_cube": (_clear_cube, [{}]), "walled_cube": (_walled_cube, [{}]),
+          "cornell": (_cornell, [{}, {"skip_cell": 1}, {"skip_cell": 3}, {"macro_cell": 4}]), "sheet": (_sheet, [{}]),
+          "vial": (_vial, [{}])}
+
+
+def _same(a, fa, b, fb, what):
+    assert a["counters"] == b["counters"], what
+    for k in ("face", "absorbed", "emitted"):
+        assert np.array_equal(a[k], b[k]), (what, k)
+    assert torch.equal(fa, fb), what
+
+
+@pytest.mark.parametrize("name", sorted(SCENES))
+@pytest.mark.parametrize("n", [1, 31, 33, 2_047, 70_001])
+def test_forms_agree_at_every_path_count(name, n):
+    require_gpu()
+    from paper_1706_03024_gb300.scene import Scene
+    make, options = SCENES[name]
+    S = Scene(make(n))
+    for opt in options:
+        # the reference: one lane per warp works, so nothing is regrouped or shared
+        one = S.render(form="wavefront", block_size=32, regroup=1, **opt).clone()
+        ref = S.read()
+        for kw in ({"form": "plain"}, {"form": "plain", "block_size": 32, "blocks_per_sm": 1}, {"form": "wavefront_warp"},
+                   {"form": "wavefront_warp", "regroup": 3}, {"form": "wavefront_warp", "block_size": 32, "blocks_per_sm": 1}):
+            f = S.render(**kw, **opt)
+            _same(S.read(), f, ref, one, (name, n, kw, opt))
+    S.close()
+
+
+@pytest.mark.parametrize("kw", [{"max_steps": 7}, {"max_events": 3}, {"n_rr": 0}, {"analog": 1}, {"max_inelastic": 1}])
+def test_ends_of_paths_agree(kw):
+    require_gpu()
+    from paper_1706_03024_gb300.scene import Scene
+    for make in (_cube, _walled_cube, _cornell):
+        S = Scene(make(5_003))
+        one = S.render(form="wavefront", block_size=32, regroup=1, **kw).clone()
+        ref = S.read()
+        for form in ("plain", "wavefront_warp"):
+            f = S.render(form=form, **kw)
+            _same(S.read(), f, ref, one, (form, kw))
+        S.close()
+
+
+@pytest.mark.parametrize("hero", [1, 2, 3, 4])
+def test_hero_forms_agree(hero):
+    require_gpu()
+    from paper_1706_03024_gb300.scene import Scene
+    for make in (_cornell, _cube):
+        S = Scene(make(4_099))
+        one = S.render(form="plain", hero=hero).clone()
+        ref = S.read()
+        f = S.render(form="wavefront_warp", hero=hero)
+        _same(S.read(), f, ref, one, hero)
+        S.close()
+
+
+@pytest.mark.parametrize("value", [0.5, 255.9999847412109, 256.0, 300.0])
+def test_fixed_point_of_large_weights(value):
+    """Tallies are sums of round(weight 2^24): a weight on either side of 2^8, where 32 bits end. An
+    uncoloured box without matter passes a source's unit weight unchanged, so the weight is made by the sum of n
+    escapes; the film value of a light seen by a sensor of tiny pixels is the large single contribution."""
+    require_gpu()
+    from paper_1706_03024_gb300.scene import Scene
+    sc = sg.cfg1_homogeneous_cube(n_paths=1, film=1)
+    edge = 1.0 / (value * 4.0 * np.pi) ** 0.5   # one isotropic vertex: 1 / (4 pi A_pix) = value
+    sc["medium"] = sg.homogeneous_medium(1, conc=0.0, sigma_s=1e4, lo=(0.0, 0.0, 0.0), hi=(1.0, 1.0, 1.0))
+    sc["sensor"] = sg.ortho_sensor(1, 1, (0.5 - edge / 2, 0.5 - edge / 2, 1.0), (edge, 0.0, 0.0), (0.0, edge, 0.0),
+                                   (0.0, 0.0, 1.0))
+    sc["params"]["max_events"] = 1
+    S = Scene(sc)
+    films = [S.render(form=f).double().cpu().numpy() for f in ("plain", "wavefront", "wavefront_warp", "wavefront_pool")]
+    for f in films:
+        assert np.array_equal(f, films[0])
+        # one contribution of value T, T = exp(-sigma depth) in (0, 1]: exact to fp32 rounding of a few operations
+        assert 0.0 < f.sum() <= value * (1.0 + 1e-5)
+    S.close()
