@@ -37,13 +37,18 @@ constexpr float TWO_PI = 6.28318530717958648f;
 // ---------------------------------------------------------------------------------------------
 // Philox4x32-10: ten rounds, each two 32x32->64 products of the even words with the round
 // multipliers, mixed with the odd words and the key; the key advances by the Weyl constants.
+__device__ __forceinline__ uint4 philox_round(uint4 c, uint32_t k0, uint32_t k1)
+{
+    const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
+    const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
+    return make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+}
+
 __device__ __forceinline__ uint4 philox(uint4 c, uint32_t k0, uint32_t k1)
 {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
-        c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+        c = philox_round(c, k0, k1);
         k0 += 0x9E3779B9u;
         k1 += 0xBB67AE85u;
     }
@@ -1064,6 +1069,26 @@ __device__ __forceinline__ Conn spawn(const M &m, const RunDev &R, const Smem &s
                       [&] { return m.rng(R, pid, STEP_SPAWN, 1u); });
 }
 
+// The same with the Philox rounds as a loop: a spawn's share of the steps is small, its share of the code is
+// not (each unrolled block is over a hundred instructions).
+template <class M>
+__device__ __forceinline__ Conn spawn_rolled(const M &m, const RunDev &R, const Smem &sm, uint64_t pid, Path &p,
+                                             int *emitter)
+{
+    uint4 c0 = make_uint4((uint32_t)pid, STEP_SPAWN, 0u, (uint32_t)(pid >> 32)), c1 = c0;
+    c1.z = 1u;
+    uint32_t k0 = R.seed, k1 = m.key1(R);
+#pragma unroll 1
+    for (int r = 0; r < 10; ++r) {
+        c0 = philox_round(c0, k0, k1);
+        c1 = philox_round(c1, k0, k1);
+        k0 += 0x9E3779B9u;
+        k1 += 0xBB67AE85u;
+    }
+    return spawn_from(m, R, sm, pid, p, emitter, U4{u24(c0.x), u24(c0.y), u24(c0.z), u24(c0.w)},
+                      [&] { return U4{u24(c1.x), u24(c1.y), u24(c1.z), u24(c1.w)}; });
+}
+
 // Decisions that need no grid read. Where a medium has grids but no solvent mask (s(x) = 1), every
 // point has sigma_t >= sigma_s + sigma_a0 (the dye terms are >= 0) and sigma_t <= sigma_bar. So a
 // tentative collision with u_real sigma_bar < sigma_s + sigma_a0 is real, and then a scatter if
@@ -1610,12 +1635,15 @@ __device__ __forceinline__ void hero_close(const M &m, HeroSet &h)
     h.isb = m.inv_maj(bm);
 }
 
+// floor(b / C) for the 1..4 wavelengths a path may carry, without a division's code.
+__device__ __forceinline__ int hero_block(int b, int C) { return C == 3 ? b / 3 : b >> (C >> 1); }
+
 // The hero's source lines: emitters first .. first + n - 1 of its source, in blocks of C.
 template <class M>
 __device__ __forceinline__ void hero_lines(const M &m, const SceneDev &S, int k, int C, HeroSet &h)
 {
     const int g0 = S.em_group_first[k], gn = S.em_group_n[k];
-    const int first = g0 + ((k - g0) / C) * C;
+    const int first = g0 + hero_block(k - g0, C) * C;
     h.n = min(C, g0 + gn - first);
     h.hero = k - first;
 #pragma unroll
@@ -1631,7 +1659,7 @@ __device__ __forceinline__ void hero_lines(const M &m, const SceneDev &S, int k,
 template <class M>
 __device__ __forceinline__ void hero_emission(const M &m, int d, int b, int C, HeroSet &h)
 {
-    const int first = (b / C) * C;
+    const int first = hero_block(b, C) * C;
     h.n = min(C, m.B() - first);
     h.hero = b - first;
     const float *cdf = m.cdf(d);
@@ -3366,17 +3394,19 @@ __device__ __forceinline__ bool hero_march_begin(const SceneDev &S, const RunDev
         if (j > 0 && j < hm.n && m.maj(hm_bin(hm, j)) > m.maj(bm)) bm = hm_bin(hm, j);
     }
     const float sb = m.maj(bm);
-    if (S.homogeneous) {
-        const MatterPt pt = matter_at(m, x);
+    if (S.homogeneous || !(sb > 0.0f)) {
+        if (S.homogeneous) {
+            const MatterPt pt = matter_at(m, x);
 #pragma unroll
-        for (int j = 0; j < HERO_MAX; ++j)
-            if (j < hm.n) hm.T[j] = __expf(-coeffs_of(m, pt, hm_bin(hm, j)).total * g.tl);
-        hero_deposit(S, R, hm);
-        return false;
-    }
-    if (!(sb > 0.0f)) {
-        hero_deposit(S, R, hm);
-        return false;
+            for (int j = 0; j < HERO_MAX; ++j)
+                if (j < hm.n) hm.T[j] = __expf(-coeffs_of(m, pt, hm_bin(hm, j)).total * g.tl);
+        }
+        hm.mc.tl = -1.0f;   // nothing to march: the first step deposits the transmittances as they are
+        hm.mc.t = 0.0f;
+        hm.mc.isb = 0.0f;
+        hm.mc.it = 0;
+        hm.mc.g = MarchRng{1u, 0u, 0u, 0u};
+        return true;
     }
     hm.mc.x = x;
     hm.mc.dir = g.dir;
@@ -3452,7 +3482,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, 4) k_trace_hero_warp(SceneDev S, R
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SmemLayout L = hero_warp_layout(S.B, blockDim.x);
     const Smem sm = block_prologue(S, smem_raw, L, R.tallies, true);
-    const MedS_<true, false> m{S, sm};
+    const MedS_<true, false, false> m{S, sm};   // hero paths have no interfaces and no glossy walls
     constexpr unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nwarps = blockDim.x >> 5;
@@ -3494,7 +3524,7 @@ __global__ void __launch_bounds__(WARP_BLOCK, 4) k_trace_hero_warp(SceneDev S, R
                     exhausted = true;
                 } else {
                     int k = 0;
-                    const Conn c = spawn(m, R, sm, R.path_offset + i, p, &k);
+                    const Conn c = spawn_rolled(m, R, sm, R.path_offset + i, p, &k);
                     hero_lines(m, S, k, R.hero, h);
                     if (c.valid) hq_push(q, c, h);
                 }
