@@ -780,8 +780,8 @@ int flr_set_sensor(flr_ctx *ctx, const flr_sensor *c)
 
 static int grow(flr_ctx *ctx, void **ptr, size_t *cap, size_t need, size_t elem, const char *what);
 
-// Zeroes the context's film accumulator for a launch over n film values (grown on demand).
-static int film_accumulator(flr_ctx *ctx, size_t n, cudaStream_t st);
+// Zeroes the context's film accumulator for a launch over `copies` copies of n film values (grown on demand).
+static int film_accumulator(flr_ctx *ctx, size_t n, int copies, cudaStream_t st);
 
 int flr_render(flr_ctx *ctx, const flr_params *p, void *stream)
 {
@@ -842,8 +842,9 @@ int flr_render(flr_ctx *ctx, const flr_params *p, void *stream)
         ctx->paths_since_clear = 0;
     }
     if (p->n_paths == 0) return FLR_OK;
+    const int copies = runs_homogeneous(S, p->form, p->n_paths, p->hero) && n_film <= FILM_COPIES_MAX_VALUES ? FILM_COPIES : 1;
     if (film_on) {
-        rc = film_accumulator(ctx, n_film, st);
+        rc = film_accumulator(ctx, n_film, copies, st);
         if (rc != FLR_OK) return rc;
     }
     e = cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), st);
@@ -863,6 +864,7 @@ int flr_render(flr_ctx *ctx, const flr_params *p, void *stream)
     R.film_scale = (float)(1.0 / (double)p->n_paths);
     R.film = film_on ? p->film : nullptr;
     R.film_fx = film_on ? ctx->d_film_fx : nullptr;
+    R.film_copies = copies;
     R.path_events = p->path_events;
     R.tallies = ctx->d_tallies;
     R.counters = ctx->d_counters;
@@ -874,7 +876,7 @@ int flr_render(flr_ctx *ctx, const flr_params *p, void *stream)
     e = launch_trace(S, R, p->form, p->block_size, p->blocks_per_sm, st);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "launch trace kernel");
     if (film_on) {
-        e = launch_film_fold(p->film, ctx->d_film_fx, n_film, p->accumulate ? 1 : 0, st);
+        e = launch_film_fold(p->film, ctx->d_film_fx, n_film, copies, p->accumulate ? 1 : 0, st);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "fold film sums");
     }
     ctx->paths_since_clear += p->n_paths;
@@ -938,7 +940,7 @@ int flr_render_camera(flr_ctx *ctx, const flr_params *p, void *stream)
         if (e != cudaSuccess) return cuda_fail(ctx, e, "clear film");
     }
     if (p->n_paths == 0) return FLR_OK;
-    rc = film_accumulator(ctx, n_film, st);
+    rc = film_accumulator(ctx, n_film, 1, st);
     if (rc != FLR_OK) return rc;
     // the kernel's block tallies are flushed into a scratch copy: the camera estimator has none
     rc = grow(ctx, (void **)&ctx->d_adj_tal, &ctx->adj_tal_cap, (size_t)tal_size(FLR_MAX_BINS),
@@ -965,7 +967,7 @@ int flr_render_camera(flr_ctx *ctx, const flr_params *p, void *stream)
     e = cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), st);
     if (e == cudaSuccess) e = launch_camera(S, R, p->form, p->block_size, st);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "launch camera kernel");
-    e = launch_film_fold(p->film, ctx->d_film_fx, n_film, p->accumulate ? 1 : 0, st);
+    e = launch_film_fold(p->film, ctx->d_film_fx, n_film, 1, p->accumulate ? 1 : 0, st);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "fold film sums");
     return FLR_OK;
 }
@@ -1280,12 +1282,12 @@ static int grow(flr_ctx *ctx, void **ptr, size_t *cap, size_t need, size_t elem,
     return FLR_OK;
 }
 
-static int film_accumulator(flr_ctx *ctx, size_t n, cudaStream_t st)
+static int film_accumulator(flr_ctx *ctx, size_t n, int copies, cudaStream_t st)
 {
-    const int rc = grow(ctx, (void **)&ctx->d_film_fx, &ctx->film_fx_cap, n, sizeof(unsigned long long),
+    const int rc = grow(ctx, (void **)&ctx->d_film_fx, &ctx->film_fx_cap, film_capacity(n), sizeof(unsigned long long),
                         "film accumulator");
     if (rc != FLR_OK) return rc;
-    const cudaError_t e = cudaMemsetAsync(ctx->d_film_fx, 0, sizeof(unsigned long long) * n, st);
+    const cudaError_t e = cudaMemsetAsync(ctx->d_film_fx, 0, sizeof(unsigned long long) * n * copies, st);
     return e == cudaSuccess ? FLR_OK : cuda_fail(ctx, e, "clear film accumulator");
 }
 

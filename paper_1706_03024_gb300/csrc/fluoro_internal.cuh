@@ -129,6 +129,7 @@ struct RunDev {
     float *film;
     unsigned long long *film_fx;       // the launch's film sums in fixed point (FILM_FX_ONE), or
                                        // NULL: contributions go to `film` by fp32 atomics
+    int film_copies;                   // copies of film_fx the launch spreads over (0 or 1: one)
     uint32_t *path_events;
     unsigned long long *tallies;       // tal_size(B)
     unsigned long long *counters;      // FLR_NCOUNTERS
@@ -220,8 +221,18 @@ int batch_occupancy_blocks_per_sm(int block);
 // so the sum does not depend on the order of the additions (up to 2^32 per film value).
 constexpr float FILM_FX_ONE = 4294967296.0f;
 constexpr double FILM_FX_INV = 1.0 / 4294967296.0;
+// Copies of the film sums that a launch may spread its additions over (RunDev::film_copies): a pencil beam puts a
+// sixth of a homogeneous cube's contributions on one film value, and additions to one address pass the L2 one
+// by one. Room for them is always held beside a small film (32 MB at most), so that no launch after the
+// first over a film size allocates.
+constexpr int FILM_COPIES = 8;
+constexpr size_t FILM_COPIES_MAX_VALUES = (size_t)1 << 19;
+inline size_t film_capacity(size_t n) { return n <= FILM_COPIES_MAX_VALUES ? n * FILM_COPIES : n; }
+// True if launch_trace runs the homogeneous medium's own kernel, which uses the copies.
+bool runs_homogeneous(const SceneDev &S, int form, uint64_t n_paths, int hero);
 // film[j] = fx[j] * 2^-32 (add = 0) or film[j] + fx[j] * 2^-32 (add = 1), j < n, through fp64.
-cudaError_t launch_film_fold(float *film, const unsigned long long *fx, size_t n, int add, cudaStream_t st);
+cudaError_t launch_film_fold(float *film, const unsigned long long *fx, size_t n, int copies, int add,
+                             cudaStream_t st);
 cudaError_t launch_trace(const SceneDev &S, const RunDev &R, int form, int block, int blocks_per_sm,
                          cudaStream_t st);
 cudaError_t launch_build_macro(const float4 *grid, float4 uniform, const uint8_t *solvent,

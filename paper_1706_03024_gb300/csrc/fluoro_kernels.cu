@@ -156,7 +156,7 @@ __device__ __forceinline__ bool check_index(bool ok, int site, long long idx)
 // 2^24 times a contribution), the result does not depend on the order of the additions, and the
 // L2 serialises integer additions to one address faster than fp32 ones. Without an accumulator
 // (the no-allocation entry point) the contribution goes to the fp32 film directly.
-__device__ __forceinline__ void film_add(const SceneDev &S, const RunDev &R, size_t idx, float val)
+__device__ __forceinline__ void film_add(const SceneDev &S, const RunDev &R, size_t idx, float val, size_t copy = 0)
 {
     if (!FLR_CHK(idx < (size_t)S.W * S.H * S.B, CK_FILM, (long long)idx)) return;
     if (R.film_fx == nullptr) {
@@ -164,7 +164,7 @@ __device__ __forceinline__ void film_add(const SceneDev &S, const RunDev &R, siz
         return;
     }
     const unsigned long long fx = __float2ull_rn(val * FILM_FX_ONE);
-    if (fx) atomicAdd(&R.film_fx[idx], fx);
+    if (fx) atomicAdd(&R.film_fx[copy + idx], fx);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -235,9 +235,9 @@ __device__ __forceinline__ void tally_add(const Smem &sm, int idx, float w)
 // MC = false compiles the local-majorant path alone out (launched whenever the scene has none:
 // the smaller code keeps the warp-regrouped kernel's loops in the instruction cache); IF = false
 // compiles dielectric faces and glossy walls out (scenes with index-matched faces and Lambertian
-// walls). LZ = true compiles in the decisions taken without a grid read (minorant_known; launched
+// walls). HOM = true compiles grids out (media without any). LZ = true compiles in the decisions taken without a grid read (minorant_known; launched
 // for media with grids and no solvent mask).
-template <bool OPT, bool MC = OPT, bool IF = true, bool LZ = false>
+template <bool OPT, bool MC = OPT, bool IF = true, bool LZ = false, bool HOM = false>
 struct MedS_ {
     static constexpr bool kLazy = LZ;
     const SceneDev &S;
@@ -249,7 +249,7 @@ struct MedS_ {
     __device__ __forceinline__ float vox_scale(int k) const { return S.vox_scale[k]; }
     __device__ __forceinline__ int dims(int k) const { return S.dims[k]; }
     __device__ __forceinline__ const int *bdims() const { return S.bdims; }
-    __device__ __forceinline__ bool homogeneous() const { return S.homogeneous != 0; }
+    __device__ __forceinline__ bool homogeneous() const { return HOM || S.homogeneous != 0; }
     __device__ __forceinline__ const float4 *grid() const { return S.grid; }
     __device__ __forceinline__ const uint8_t *solvent() const { return S.solvent; }
     __device__ __forceinline__ float4 conc_uniform() const
@@ -1472,6 +1472,14 @@ __host__ __device__ inline SmemLayout smem_layout(int B, int form, int block)
     return L;
 }
 
+// The homogeneous medium's kernel: tables and counters only, tallies in global memory.
+__host__ __device__ inline SmemLayout homogeneous_layout(int B)
+{
+    SmemLayout L = smem_layout(B, FLR_FORM_WAVEFRONT_WARP, 0);
+    L.total_bytes = L.queue_off_bytes;
+    return L;
+}
+
 __device__ __forceinline__ Smem block_prologue(const SceneDev &S, unsigned char *raw, const SmemLayout &L,
                                                unsigned long long *global_tal, bool persistent = false)
 {
@@ -2370,11 +2378,10 @@ __global__ void __launch_bounds__(256) k_frozen_sums(SceneDev S, RunDev R, PertD
 // ---------------------------------------------------------------------------------------------
 // Wavefront form with per-warp regrouping and pull-based connection drains. Each warp queues its
 // lanes' sensor connections in shared memory (up to WQ_CAP records). Once WQ_DRAIN records are
-// waiting (or the work is done) the warp drains the queue (wq_drain): records are begun 32 together,
-// then every lane advances its own ratio-tracking march by one step per iteration and takes the next one
-// as soon as its march ends. Against claims of single records in every iteration, and spawns of eight
-// lanes apart from the tracking step: the light sheet 186.7 -> 171.2 ms, the Cornell box 11.5 -> 10.5 ms (a
-// preview of 97 x 71 pixels 1.14 -> 0.92), a fit step 17.5 -> 17.2 ms. The marches consume their random numbers exactly as transmittance() does, so
+// waiting (or the work is done) the warp drains the queue: every lane advances its own
+// ratio-tracking march by one step per iteration and claims the next record as soon as its march
+// ends, so the lanes stay busy until the queue runs dry instead of waiting for the longest march
+// of a fixed batch. The marches consume their random numbers exactly as transmittance() does, so
 // every launch form gives the same film up to the order of the fp32 film atomics.
 //
 // The same kernel runs the two passes of the adjoint replay (MODE):
@@ -2826,6 +2833,59 @@ __global__ void __launch_bounds__(256) k_trace_plain(SceneDev S, RunDev R)
         for (int k = 0; k < PLAIN_MARCH && marching; ++k)
             marching = march_advance<WM_RENDER, LZ>(S, R, sm, A, mc, rc) &&
                        march_matter<WM_RENDER, LZ>(S, R, sm, A, mc, rc, gsig);
+    }
+    block_epilogue(S, R, sm, rc);
+}
+
+// ---------------------------------------------------------------------------------------------
+// The warp form of a homogeneous medium with index-matched faces and Lambertian walls. There nearly every
+// step of a lane ends in a vertex, and a vertex's transmittance is closed (Eq. 6): nothing is to be regrouped,
+// so each lane connects its vertex at once, without queues, marches or the generators they seed (71 registers,
+// seven blocks an SM). It was then bound by the film's hottest value (without film additions 13.0 ms instead of 16.7,
+// whatever the blocks), so a small film's sums are spread over FILM_COPIES copies, which the fold adds up. The
+// cube of a pencil beam, 20,000,000 paths: 17.3 -> 13.4 ms on a 64 x 64 film, 15.2 on a 256 x 256 one (no copies); 4,000,000:
+// 3.97 -> 3.38. A small launch lasts as long as its longest path, which here waits for its own connections:
+// 10,000 paths 0.41 -> 0.52 ms, 250,000 0.86 -> 1.02, 1,000,000 1.45 -> 1.47. Hence HOMOGENEOUS_MIN; below it, and
+// with interfaces, the queued kernel runs. `regroup` has no meaning here.
+constexpr unsigned long long HOMOGENEOUS_MIN = 1ull << 20;
+
+__global__ void __launch_bounds__(WARP_BLOCK, 7) k_trace_homogeneous(SceneDev S, RunDev R)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ PathIds s_ids[WARP_BLOCK / 32];
+    const SmemLayout L = homogeneous_layout(S.B);
+    const Smem sm = block_prologue(S, smem_raw, L, R.tallies, true);
+    const MedS_<false, false, false, false, true> m{S, sm};
+    constexpr unsigned FULL = 0xffffffffu;
+    const size_t copy = R.film_copies > 1 ? (size_t)(blockIdx.x % R.film_copies) * S.W * S.H * S.B : 0;
+    PathIds *const ids = &s_ids[threadIdx.x >> 5];
+    if ((threadIdx.x & 31) == 0) *ids = PathIds{0ull, 0, 0};
+    __syncwarp();
+    RegCnt rc = {0, 0, 0, 0, 0, 0, 0};
+    Path p;
+    p.alive = false;
+    for (uint32_t round = 1;; ++round) {
+        if (round % CARRY_ROUNDS == 0u) counters_carry(sm);
+        const unsigned need = __ballot_sync(FULL, !p.alive);
+        if (need != 0u) {
+            if (ids_left(ids)) {
+                if (__popc(need) >= CLAIM_MIN || need == FULL) {
+                    unsigned long long i;
+                    if (claim_path(ids, R, need, i)) path_claimed(p, R.path_offset + i);
+                }
+            } else if (need == FULL) {
+                break;
+            }
+        }
+        if (!p.alive) continue;
+        const Conn c = spawn_or_track(m, R, sm, p, rc);
+        if (!c.valid) continue;
+        const ConnGeom g = connect_geom(S, sm, c.x, c.lamb);
+        if (!g.ok) continue;
+        rc.connections++;
+        const float T = m.maj(c.bin) > 0.0f ? __expf(-sigma_t_at(m, c.x, c.bin) * g.tl) : 1.0f;
+        const float val = c.w * g.gf * T * R.film_scale;
+        if (val > 0.0f) film_add(S, R, (size_t)g.pix * S.B + c.bin, val, copy);
     }
     block_epilogue(S, R, sm, rc);
 }
@@ -4267,21 +4327,27 @@ __global__ void k_sample_emission(const float *__restrict__ cdf, int B, const fl
         out[i] = sample_cdf(cdf, B, u[i]);
 }
 
-// Folds a launch's fixed-point film sums into the fp32 film: film[j] = fx[j] 2^-32, or
+// Folds a launch's fixed-point film sums (of all its copies) into the fp32 film: film[j] = fx[j] 2^-32, or
 // film[j] + fx[j] 2^-32 when the launch adds to the film (one fp32 rounding per value and launch).
-// Two values per thread and iteration as 16-byte loads of the sums when both buffers allow it.
+// Two values per thread and iteration as 16-byte loads of the sums when the buffers allow it.
 __global__ void __launch_bounds__(256) k_film_fold(float *__restrict__ film,
                                                    const unsigned long long *__restrict__ fx,
-                                                   long long n, int add)
+                                                   long long n, int copies, int add)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool vec = ((reinterpret_cast<uintptr_t>(film) & 7) | (reinterpret_cast<uintptr_t>(fx) & 15)) == 0;
+    const bool vec = ((reinterpret_cast<uintptr_t>(film) & 7) | (reinterpret_cast<uintptr_t>(fx) & 15)) == 0 &&
+                     (copies == 1 || n % 2 == 0);
     long long done = 0;
     if (vec) {
         const long long pairs = n / 2;
         for (long long i = first; i < pairs; i += stride) {
-            const ulonglong2 v = __ldcs(reinterpret_cast<const ulonglong2 *>(fx) + i);
+            ulonglong2 v = __ldcs(reinterpret_cast<const ulonglong2 *>(fx) + i);
+            for (int c = 1; c < copies; ++c) {
+                const ulonglong2 w = __ldcs(reinterpret_cast<const ulonglong2 *>(fx) + c * pairs + i);
+                v.x += w.x;
+                v.y += w.y;
+            }
             float2 f = make_float2((float)((double)v.x * FILM_FX_INV), (float)((double)v.y * FILM_FX_INV));
             float2 *o = reinterpret_cast<float2 *>(film) + i;
             if (add) {
@@ -4294,7 +4360,9 @@ __global__ void __launch_bounds__(256) k_film_fold(float *__restrict__ film,
         done = pairs * 2;
     }
     for (long long j = done + first; j < n; j += stride) {
-        const float f = (float)((double)fx[j] * FILM_FX_INV);
+        unsigned long long v = fx[j];
+        for (int c = 1; c < copies; ++c) v += fx[c * n + j];
+        const float f = (float)((double)v * FILM_FX_INV);
         film[j] = add ? film[j] + f : f;
     }
 }
@@ -4449,11 +4517,30 @@ cudaError_t launch_pool(const SceneDev &S, const RunDev &R, int blocks_per_sm, c
     return cudaGetLastError();
 }
 
+bool runs_homogeneous(const SceneDev &S, int form, uint64_t n_paths, int hero)
+{
+    return form == FLR_FORM_WAVEFRONT_WARP && hero == 0 && S.homogeneous && !S.iface && n_paths >= HOMOGENEOUS_MIN;
+}
+
+cudaError_t launch_homogeneous(const SceneDev &S, const RunDev &R, int block, int blocks_per_sm, cudaStream_t st)
+{
+    block = block <= 0 ? WARP_BLOCK : std::min(block, WARP_BLOCK);
+    const auto k = k_trace_homogeneous;
+    const int smem = homogeneous_layout(S.B).total_bytes;
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, block, smem);
+    if (occ < 1) occ = 1;
+    if (blocks_per_sm <= 0 || blocks_per_sm > occ) blocks_per_sm = occ;
+    k<<<(unsigned)(num_sms() * blocks_per_sm), block, smem, st>>>(S, R);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_trace(const SceneDev &S, const RunDev &R, int form, int block, int blocks_per_sm,
                          cudaStream_t st)
 {
     if (form == FLR_FORM_WAVEFRONT_POOL) return launch_pool(S, R, blocks_per_sm, st);
     if (R.hero > 0 && form == FLR_FORM_WAVEFRONT_WARP) return launch_hero_warp(S, R, block, blocks_per_sm, st);
+    if (runs_homogeneous(S, form, R.n_paths, R.hero)) return launch_homogeneous(S, R, block, blocks_per_sm, st);
     if (block <= 0) block = trace_block_default();
     if (form == FLR_FORM_WAVEFRONT_WARP) block = std::min(block, WARP_BLOCK);
     const int smem = trace_smem_bytes(S.B, form, block);
@@ -4698,14 +4785,15 @@ cudaError_t launch_debug_sigma_t(const SceneDev &S, const float *pts, long long 
     return cudaGetLastError();
 }
 
-cudaError_t launch_film_fold(float *film, const unsigned long long *fx, size_t n, int add, cudaStream_t st)
+cudaError_t launch_film_fold(float *film, const unsigned long long *fx, size_t n, int copies, int add,
+                             cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
     long long blocks = ((long long)n / 2 + 255) / 256;
     const long long cap = (long long)num_sms() * 8;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    k_film_fold<<<(unsigned)blocks, 256, 0, st>>>(film, fx, (long long)n, add);
+    k_film_fold<<<(unsigned)blocks, 256, 0, st>>>(film, fx, (long long)n, copies, add);
     return cudaGetLastError();
 }
 

@@ -97,6 +97,27 @@ def test_hero_forms_agree(hero):
         S.close()
 
 
+@pytest.mark.parametrize("film", [16, 17, 80, 81])   # even, odd; the largest with copies of its sums, the first without
+@pytest.mark.parametrize("n", [(1 << 20) - 1, 1 << 20, (1 << 20) + 33])
+def test_homogeneous_kernel(n, film):
+    """From 2^20 paths on the warp form of a homogeneous medium runs a kernel of its own."""
+    require_gpu()
+    from paper_1706_03024_gb300.scene import Scene
+    for medium in (None, sg.homogeneous_medium(1, conc=0.5, sigma_s=5.0, sigma_a0=0.3, wall_mask=0b011111, wall_albedo=0.9)):
+        sc = sg.cfg1_homogeneous_cube(n_paths=n, film=film)
+        if medium is not None:
+            sc["medium"] = medium
+        S = Scene(sc)
+        one = S.render(form="plain").clone()
+        ref = S.read()
+        for kw in ({}, {"block_size": 32, "blocks_per_sm": 2}):
+            f = S.render(form="wavefront_warp", **kw)
+            _same(S.read(), f, ref, one, (n, film, kw))
+        f = S.render(form="wavefront_warp", accumulate=True)   # the second launch adds the same sums once more
+        assert torch.equal(f, one + one)
+        S.close()
+
+
 @pytest.mark.parametrize("value", [0.5, 255.9999847412109, 256.0, 300.0])
 def test_fixed_point_of_large_weights(value):
     """Tallies are sums of round(weight 2^24): a weight on either side of 2^8, where 32 bits end. An
