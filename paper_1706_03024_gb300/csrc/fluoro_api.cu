@@ -704,17 +704,13 @@ static int set_medium_on(flr_ctx *ctx, const flr_medium *m, cudaStream_t st, boo
             }
             ctx->grid_cap = np;
         }
-        e = launch_pack_grid(mm.conc, mm.conc_uniform, mm.n_dyes, mm.dims, ctx->d_grid, st);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "pack grids");
     }
-    bool any_grid = false;
-    for (int d = 0; d < mm.n_dyes; ++d) any_grid = any_grid || mm.conc[d];
-    if (any_grid || mm.solvent) {
+    if (grids) {
         unsigned int h[MAXD + 2] = {0, 0, 0, 0, 0, 0};
         e = cudaMemsetAsync(ctx->d_scratch, 0, sizeof(h), st);
-        for (int d = 0; d < mm.n_dyes && e == cudaSuccess; ++d)
-            if (mm.conc[d])
-                e = launch_grid_max(mm.conc[d], n, ctx->d_scratch + d, (int *)(ctx->d_scratch + MAXD), st);
+        if (e == cudaSuccess && medium_has_grid(mm))
+            e = launch_pack_grid_max(mm.conc, mm.conc_uniform, mm.n_dyes, mm.dims, ctx->d_grid, ctx->d_scratch,
+                                     (int *)(ctx->d_scratch + MAXD), st);
         if (e == cudaSuccess && mm.solvent) e = launch_solvent_any(mm.solvent, n, ctx->d_scratch + MAXD + 1, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h, ctx->d_scratch, sizeof(h), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);

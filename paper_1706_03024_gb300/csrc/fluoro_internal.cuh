@@ -246,6 +246,9 @@ cudaError_t launch_grid_max(const float *g, long long n, unsigned int *out_bits,
 // interleaves the dyes' row-major grids into the bricked layout (packed_voxels(dims) float4s)
 cudaError_t launch_pack_grid(const float *const *conc, const float *uniform, int D, const int dims[3],
                              float4 *out, cudaStream_t st);
+// the same, with the maxima of the given grids (bit patterns, zeroed by the caller) and a flag for bad values
+cudaError_t launch_pack_grid_max(const float *const *conc, const float *uniform, int D, const int dims[3], float4 *out,
+                                 unsigned int *max_bits, int *neg_flag, cudaStream_t st);
 cudaError_t launch_solvent_any(const uint8_t *s, long long n, unsigned int *out, cudaStream_t st);
 cudaError_t launch_philox(uint32_t seed, uint32_t medium, const uint32_t *ctr, long long n,
                           uint32_t *out, cudaStream_t st);

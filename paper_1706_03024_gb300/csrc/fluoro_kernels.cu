@@ -4259,6 +4259,8 @@ __global__ void k_dist_init(const float4 *__restrict__ mc, const float *__restri
     }
 }
 
+// Distances along one axis, outward from each cell: no cell at distance a can lower a best of at most a, so
+// the search ends at the nearest matter instead of visiting all 2 cap cells around.
 __global__ void k_dist_axis(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int mx, int my,
                             int mz, int axis, int cap)
 {
@@ -4267,15 +4269,13 @@ __global__ void k_dist_axis(const uint8_t *__restrict__ in, uint8_t *__restrict_
     const long long stride = axis == 0 ? 1 : (axis == 1 ? mx : (long long)mx * my);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
-        const int c = axis == 0 ? (int)(i % mx) : (axis == 1 ? (int)((i / mx) % my) : (int)(i / ((long long)mx * my)));
-        int best = in[i];
-        const int lo = max(-cap, -c), hi = min(cap, len - 1 - c);
-        for (int k = lo; k <= hi; ++k) {
-            const int a = k < 0 ? -k : k;
-            if (a >= best) continue;   // max(|k|, .) cannot beat the best so far
-            best = min(best, max(a, (int)in[i + k * stride]));
+        const int c = n <= 0xFFFFFFFFll ? (int)((uint32_t)i / (uint32_t)stride % (uint32_t)len) : (int)(i / stride % len);
+        int best = min((int)in[i], cap);
+        for (int a = 1; a < best; ++a) {
+            if (a <= c) best = min(best, max(a, (int)in[i - a * stride]));
+            if (a < len - c) best = min(best, max(a, (int)in[i + a * stride]));
         }
-        out[i] = (uint8_t)min(best, cap);
+        out[i] = (uint8_t)best;
     }
 }
 
@@ -4299,6 +4299,44 @@ __global__ void k_pack_grid(PackArgs a, long long n, float4 *__restrict__ out)
         const int ix = (int)(i % a.dims[0]), iy = (int)((i / a.dims[0]) % a.dims[1]);
         const int iz = (int)(i / ((long long)a.dims[0] * a.dims[1]));
         out[packed_index(ix, iy, iz, a.bdims)] = make_float4(v[0], v[1], v[2], v[3]);
+    }
+}
+
+// The same with the largest value of each given grid (and a flag for negative or non-finite ones): one pass
+// over the grids where the packing and a pass of maxima for each dye made two, and one atomic a
+// block where those made one a warp.
+__global__ void __launch_bounds__(256) k_pack_grid_max(PackArgs a, uint32_t n, float4 *__restrict__ out,
+                                                       unsigned int *__restrict__ max_bits, int *neg_flag)
+{
+    __shared__ float s_max[8][MAXD];
+    float m[MAXD] = {0.f, 0.f, 0.f, 0.f};
+    bool bad = false;
+    const uint32_t nx = a.dims[0], nxy = nx * (uint32_t)a.dims[1];
+    for (unsigned long long j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+        const uint32_t i = (uint32_t)j;
+        float v[MAXD] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int d = 0; d < MAXD; ++d) {
+            if (d >= a.D) continue;
+            v[d] = a.conc[d] ? a.conc[d][i] : a.uniform[d];
+            if (!a.conc[d]) continue;
+            if (!(v[d] >= 0.0f) || !isfinite(v[d])) bad = true; else m[d] = fmaxf(m[d], v[d]);
+        }
+        const uint32_t iz = i / nxy, r = i - iz * nxy, iy = r / nx;
+        out[packed_index((int)(r - iy * nx), (int)iy, (int)iz, a.bdims)] = make_float4(v[0], v[1], v[2], v[3]);
+    }
+#pragma unroll
+    for (int d = 0; d < MAXD; ++d) {
+        // values are not negative: their bits are ordered as they are
+        const unsigned b = __reduce_max_sync(0xffffffffu, __float_as_uint(m[d]));
+        if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5][d] = __uint_as_float(b);
+    }
+    const int any_bad = __syncthreads_or(bad);
+    if (threadIdx.x < MAXD) {
+        float t = 0.0f;
+        for (int w = 0; w < 8; ++w) t = fmaxf(t, s_max[w][threadIdx.x]);
+        if (t > 0.0f) atomicMax(&max_bits[threadIdx.x], __float_as_uint(t));
+        if (threadIdx.x == 0 && any_bad) atomicOr(neg_flag, 1);
     }
 }
 
@@ -4726,6 +4764,25 @@ cudaError_t launch_pack_grid(const float *const *conc, const float *uniform, int
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     k_pack_grid<<<(unsigned)blocks, 256, 0, st>>>(a, n, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pack_grid_max(const float *const *conc, const float *uniform, int D, const int dims[3], float4 *out,
+                                 unsigned int *max_bits, int *neg_flag, cudaStream_t st)
+{
+    PackArgs a;
+    for (int d = 0; d < MAXD; ++d) {
+        a.conc[d] = d < D ? conc[d] : nullptr;
+        a.uniform[d] = d < D ? uniform[d] : 0.0f;
+    }
+    a.D = D;
+    for (int k = 0; k < 3; ++k) {
+        a.dims[k] = dims[k];
+        a.bdims[k] = grid_bricks(dims[k]);
+    }
+    const long long n = (long long)dims[0] * dims[1] * dims[2];
+    const long long blocks = std::max(1ll, std::min((n + 255) / 256, (long long)num_sms() * 8));
+    k_pack_grid_max<<<(unsigned)blocks, 256, 0, st>>>(a, (uint32_t)n, out, max_bits, neg_flag);
     return cudaGetLastError();
 }
 

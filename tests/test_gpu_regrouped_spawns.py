@@ -138,3 +138,39 @@ def test_fixed_point_of_large_weights(value):
         # one contribution of value T, T = exp(-sigma depth) in (0, 1]: exact to fp32 rounding of a few operations
         assert 0.0 < f.sum() <= value * (1.0 + 1e-5)
     S.close()
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (3, 5, 2), (33, 17, 65), (4, 70, 9)])
+def test_upload_reads_every_voxel_and_every_distance(dims):
+    """The upload's maxima bound the majorant (a voxel above it would be counted) and refuse a bad value in any
+    voxel; the empty-space distances change neither the film's expectation nor, in what leaps nowhere, a bit."""
+    require_gpu()
+    from paper_1706_03024_gb300.scene import Scene
+    nx, ny, nz = dims
+    rng = np.random.default_rng(nx * 100 + ny)
+    n = nx * ny * nz
+    for at in (0, n - 1, n // 2):
+        conc = np.zeros((1, nz, ny, nx), np.float32)
+        conc.reshape(-1)[at] = 7.0   # one voxel holds all the dye: the maximum is there
+        sc = sg.cfg1_homogeneous_cube(n_paths=20_000, film=8)
+        sc["medium"] = sg.grid_medium(conc, sigma_s=0.0)
+        S = Scene(sc)
+        films = []
+        for kw in ({}, {"skip_cell": 1}):
+            for form in ("plain", "wavefront", "wavefront_warp"):
+                f = S.render(form=form, **kw).clone()
+                r = S.read()
+                assert r["counters"]["majorant_violations"] == 0
+                films.append((f, r))
+            for f, r in films[-3:]:
+                assert torch.equal(f, films[-3][0]) and r["counters"] == films[-3][1]["counters"]
+        # leaps draw other random numbers: the same expected escapes
+        a, b = (x[1]["face"].sum() for x in (films[0], films[3]))
+        assert abs(a - b) <= 6.0 * (2 * 0.25 / 20_000) ** 0.5   # weights in [0, 1]: variance at most 1/4 each
+        S.close()
+        for bad in (-1.0, np.nan, np.inf):
+            worse = rng.uniform(0.0, 1.0, conc.shape).astype(np.float32)
+            worse.reshape(-1)[at] = bad
+            sc["medium"] = sg.grid_medium(worse, sigma_s=0.0)
+            with pytest.raises(Exception, match="negative or non-finite"):
+                Scene(sc)
