@@ -1423,7 +1423,8 @@ struct SmemLayout {
 // Per-warp connection queue of the warp-regrouped form: capacity and drain threshold. A drain starts
 // once WQ_DRAIN records wait; one tracking round adds at most 32, so the queue never wraps. A drain begins
 // its records 32 together and keeps its unfinished marches (wq_drain), so it has no tail to spread over a longer
-// queue: 128 records measured as 224 (the light sheet 171.2 and 171 ms, the Cornell box 10.5 and 10.6).
+// queue: 128 records measured as 224 (the light sheet 181.9 and 180.3 ms, the Cornell box 10.85 and 11.01, its
+// preview 0.94 and 0.97, all before the queue records were shortened).
 // Four blocks of 128 threads (at most 128 registers) share an SM: with five (96 registers) the two kinds of
 // work of a drain spill in their loops, and every workload took 20 to 60 % longer.
 constexpr int WARP_BLOCK = 128;   // threads per block of the warp-regrouped form
@@ -1432,7 +1433,7 @@ constexpr int WQ_CAP = 128;
 constexpr int WQ_DRAIN = WQ_CAP - 32;
 constexpr int MS_CAP = 64;        // stack of marches that wait: fewer than 32 before 32 records are begun
 constexpr int MS_WORDS = 19;      // 4-byte fields per waiting march
-constexpr int DRAIN_KEEP = 16;    // a drain ends once fewer lanes would go on (8 and 24 measured the same)
+constexpr int DRAIN_KEEP = 16;    // a drain ends once fewer lanes would go on (24: 226 for 229 ms on the sheet, more on the box)
 constexpr int SPAWN_MIN = 8;      // lanes that start new paths together (hero, camera; pass 2 of the adjoint)
 constexpr int CLAIM_MIN = 4;      // lanes that take path ids together (the light sheet: 1: 180, 4: 182, 8: 189 ms)
 constexpr int WARP_WORDS = 6;     // head, tail and PathIds of a warp (8-byte aligned)
@@ -2797,8 +2798,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, WARP_BLOCKS) k_trace_wavefront_war
 // its own path. A thread is either tracking or inside a connection's march; every iteration of the warp
 // gives the tracking lanes one step and the marching lanes up to PLAIN_MARCH. With the march as a loop inside the
 // step, all lanes of a warp waited at every step for the longest of its marches: render()'s defaults on the
-// 100 x 100 Cornell box, 10 paths a pixel, took 3.97 ms instead of 3.19 (2 and 6 march steps: 3.19 and 3.42), the
-// 4.2 million paths of the 512 x 512 one 101 instead of 42 ms, an eighth of the full light sheet 171 instead of 42.
+// 100 x 100 Cornell box, 10 paths a pixel, took 3.97 ms instead of 3.19 (2 and 6 march steps: 3.19 and 3.42), with the
+// step's smaller code the 4.2 million paths of the 512 x 512 one went from 101 to 42 ms, an eighth of the light sheet from 171 to 42.
 constexpr int PLAIN_MARCH = 3;
 
 template <bool OPT, bool IF, bool LZ = false>
