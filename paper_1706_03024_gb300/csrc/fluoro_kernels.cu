@@ -1413,6 +1413,17 @@ __device__ __forceinline__ bool claim_path(PathIds *ids, const RunDev &R, unsign
     return ((need >> lane) & 1u) && rank < left;
 }
 
+// The length of a warp's queue, called by the whole warp after its pushes. The first __syncwarp shows every lane the records,
+// the second keeps a lane's next push behind the other lanes' reads: the votes between the rounds order
+// execution, not memory, and lanes that read different lengths would disagree about draining.
+__device__ __forceinline__ int queue_length(const int *tail)
+{
+    __syncwarp();
+    const int n = *tail;
+    __syncwarp();
+    return n;
+}
+
 // ---------------------------------------------------------------------------------------------
 // Block prologue / epilogue: stage tables, zero and flush block tallies and counters.
 struct SmemLayout {
@@ -2772,9 +2783,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, WARP_BLOCKS) k_trace_wavefront_war
             pre += a;
             if (a != 0.0f) { wq_push(q, p, a, c.lamb, 0); break; }
         }
-        __syncwarp();
+        const int avail = queue_length(&q.head_tail[1]);
         const bool any = __any_sync(FULL, p.alive) || ids_left(ids);
-        const int avail = q.head_tail[1];
         if (avail >= WQ_DRAIN || (!any && avail + q.head_tail[0] > 0))
             wq_drain<MODE, MC, LZ>(S, R, sm, A, q, stack, avail, !any, rc, gsig);
         if (!any) break;
@@ -3595,9 +3605,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, 4) k_trace_hero_warp(SceneDev S, R
             const Conn c = track_step_hero(m, R, sm, p, h, rc);
             if (c.valid) hq_push(q, c, h);
         }
-        __syncwarp();
+        const int avail = queue_length(&q.head_tail[1]);
         const bool any = __any_sync(FULL, p.alive || !exhausted);
-        const int avail = q.head_tail[1];
         if (avail >= HQ_DRAIN || (!any && avail > 0)) {
             HMarch hm;
             bool active = false;
@@ -4013,9 +4022,8 @@ __global__ void __launch_bounds__(256, 2) k_trace_camera_warp(SceneDev S, RunDev
                 f[12 * CQ_CAP] = __uint_as_float(step);
             }
         }
-        __syncwarp();
+        const int avail = queue_length(tail);
         const bool any = __any_sync(FULL, cp.alive || !exhausted);
-        const int avail = *tail;
         if (avail >= CQ_DRAIN || (!any && avail > 0)) {
             // pull-based drain; claims every second iteration (see the light tracer's warp form)
             float3 x0, dir;
