@@ -2681,6 +2681,7 @@ __device__ __forceinline__ void wq_drain(const SceneDev &S, const RunDev &R, con
             active = true;
         }
         depth = max(depth - n_idle, 0);
+        __syncwarp();   // the slots just read may be written from here on: the votes alone would not order the two
         const unsigned act = __ballot_sync(FULL, active);
         if (act == 0u) break;
         if (avail < least && depth == 0 && !last && __popc(act) < DRAIN_KEEP) {

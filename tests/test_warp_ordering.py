@@ -1,8 +1,8 @@
-"""Memory ordering of the warp-regrouped kernels' shared queues. The lanes of a warp pass records to one
+"""Memory ordering of the warp-regrouped kernels' shared queues and stacks. The lanes of a warp pass records to one
 another through shared memory; a vote (ballot, any) orders their execution but not their memory, only __syncwarp does
 both. Here the kernels' own source runs on the host, 32 threads for the lanes, under a race detector that
 knows the difference (tests/hostwarp/warp.h); it also checks that every connection is made exactly once and that no
-queue index leaves its bounds."""
+queue or stack index leaves its bounds."""
 import os
 import re
 import subprocess
@@ -62,16 +62,31 @@ def _program(kernel):
                            ["SPAWN_MIN", "CARRY_ROUNDS", "CQ_CAP", "CQ_DRAIN", "CQ_WORDS"])
         body = [inc("camera.h"), *const, *d.values()]
         return body, MAIN.replace("RUN", "").replace("CALL", "k_trace_camera_warp(SceneDev{}, R)")
-    const, d = _source(LIGHT + [_f("queue_length"), r"struct HQueue\b", _f("hq_push"), _f("k_trace_hero_warp", "__global__ void")],
-                       ["WARP_BLOCK", "SPAWN_MIN", "CARRY_ROUNDS", "HERO_MAX", "HQ_CAP", "HQ_DRAIN", "HQ_WORDS"])
+    const = ["WARP_BLOCK", "SPAWN_MIN", "CARRY_ROUNDS"]
+    if kernel == "hero":
+        const, d = _source(LIGHT + [_f("queue_length"), r"struct HQueue\b", _f("hq_push"),
+                                    _f("k_trace_hero_warp", "__global__ void")],
+                           const + ["HERO_MAX", "HQ_CAP", "HQ_DRAIN", "HQ_WORDS"])
+        d = list(d.values())
+        n = len(LIGHT)
+        body = [inc("light.h"), "constexpr uint32_t STEP_SPAWN = 0xFFFFFFFFu;\n", *const, *d[:n], inc("light_model.h"),
+                inc("hero.h"), *d[n:n + 3], inc("hero_main.h"), *d[n + 3:]]
+        return body, MAIN.replace("RUN", "R.hero = 4;").replace("CALL", "k_trace_hero_warp(SceneDev{}, R)")
+    const, d = _source(LIGHT + [r"struct PathIds\b", _f("wq_push"), _f("ids_left"), _f("queue_length"), _f("claim_path"),
+                                _f("path_claimed"), _f("stack_store"), _f("stack_load"), _f("wq_drain"),
+                                _f("k_trace_wavefront_warp", "__global__ void")],
+                       const + ["WARP_BLOCKS", "WQ_CAP", "WQ_DRAIN", "MS_CAP", "MS_WORDS", "DRAIN_KEEP", "CLAIM_MIN",
+                                "WARP_WORDS", "MAX_REGROUP", "WM_RENDER", "WM_ADJ_WEIGHTS", "WM_ADJ_GRAD", "WQ_ORD_MAX"])
     d = list(d.values())
     n = len(LIGHT)
     body = [inc("light.h"), "constexpr uint32_t STEP_SPAWN = 0xFFFFFFFFu;\n", *const, *d[:n], inc("light_model.h"),
-            inc("hero.h"), *d[n:n + 3], inc("hero_main.h"), *d[n + 3:]]
-    return body, MAIN.replace("RUN", "R.hero = 4;").replace("CALL", "k_trace_hero_warp(SceneDev{}, R)")
+            inc("warp_main.h"), *d[n:]]
+    regroup = kernel.split("/")[1]
+    return body, MAIN.replace("RUN", f"R.regroup = {regroup};").replace(
+        "CALL", "k_trace_wavefront_warp<WM_RENDER, false, false, true>(SceneDev{}, R, AdjDev{})")
 
 
-@pytest.mark.parametrize("kernel", ["hero", "camera"])
+@pytest.mark.parametrize("kernel", ["light/1", "light/3", "hero", "camera"])
 def test_lanes_exchange_records_only_across_a_syncwarp(tmp_path, kernel):
     body, main = _program(kernel)
     src, exe = tmp_path / "warp.cpp", tmp_path / "warp"
