@@ -223,11 +223,15 @@ constexpr float FILM_FX_ONE = 4294967296.0f;
 constexpr double FILM_FX_INV = 1.0 / 4294967296.0;
 // Copies of the film sums that a launch may spread its additions over (RunDev::film_copies): a pencil beam puts a
 // sixth of a homogeneous cube's contributions on one film value, and additions to one address pass the L2 one
-// by one. Room for them is always held beside a small film (32 MB at most), so that no launch after the
-// first over a film size allocates.
+// by one. Room for them is held beside every film (32 MB at most). The capacity never falls as the film
+// grows, so a context that has rendered a film allocates nothing for a smaller one, and its launches can be captured.
 constexpr int FILM_COPIES = 8;
 constexpr size_t FILM_COPIES_MAX_VALUES = (size_t)1 << 19;
-inline size_t film_capacity(size_t n) { return n <= FILM_COPIES_MAX_VALUES ? n * FILM_COPIES : n; }
+inline size_t film_capacity(size_t n)
+{
+    const size_t with_copies = (n < FILM_COPIES_MAX_VALUES ? n : FILM_COPIES_MAX_VALUES) * FILM_COPIES;
+    return n > with_copies ? n : with_copies;
+}
 // True if launch_trace runs the homogeneous medium's own kernel, which uses the copies.
 bool runs_homogeneous(const SceneDev &S, int form, uint64_t n_paths, int hero);
 // film[j] = fx[j] * 2^-32 (add = 0) or film[j] + fx[j] * 2^-32 (add = 1), j < n, through fp64.
