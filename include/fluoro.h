@@ -251,8 +251,8 @@ int flr_set_sensor(flr_ctx *ctx, const flr_sensor *sensor);
  * accumulate inside the context (read them with flr_read_tallies); film contributions, already
  * divided by p->n_paths, are summed exactly in 64-bit fixed point (units of 2^-32; at most 2^32
  * per film value and launch) in a context buffer (8 bytes per film value, or 64 per
- * value of the first 2^19 where that is more; allocated on the first launch with a film and again only
- * for a larger film), then written to p->film (accumulate = 0) or added to it when the
+ * value of the first 2^19 where that is more and to be had; allocated on the first launch with a film
+ * and again only for a larger film), then written to p->film (accumulate = 0) or added to it when the
  * launch ends: the film does not depend on the order of the contributions. Every form traces the
  * same paths (Sec. 3, Eq. 12; fixed-point tallies identical bit for bit). For a
  * medium with grids, no solvent mask and sigma_s + sigma_a0 at least 0.9 of every bin's majorant,

@@ -65,6 +65,7 @@ struct flr_ctx {
     size_t adj_tal_cap = 0;
     unsigned long long *d_film_fx = nullptr;  // a launch's film sums in fixed point (film-sized)
     size_t film_fx_cap = 0;
+    size_t film_fx_values = 0;                // the largest film it was grown for
     uint64_t paths_since_clear = 0;
     std::vector<float> h_tables;
     // local majorants of the current medium (built on demand for one cell size)
@@ -776,8 +777,9 @@ int flr_set_sensor(flr_ctx *ctx, const flr_sensor *c)
 
 static int grow(flr_ctx *ctx, void **ptr, size_t *cap, size_t need, size_t elem, const char *what);
 
-// Zeroes the context's film accumulator for a launch over `copies` copies of n film values (grown on demand).
-static int film_accumulator(flr_ctx *ctx, size_t n, int copies, cudaStream_t st);
+// Zeroes the context's film accumulator for a launch over `copies` copies of n > 0 film values. It is grown for the
+// largest film so far; where the memory for all copies is not to be had, `copies` is cut to what there is.
+static int film_accumulator(flr_ctx *ctx, size_t n, int &copies, cudaStream_t st);
 
 int flr_render(flr_ctx *ctx, const flr_params *p, void *stream)
 {
@@ -838,7 +840,7 @@ int flr_render(flr_ctx *ctx, const flr_params *p, void *stream)
         ctx->paths_since_clear = 0;
     }
     if (p->n_paths == 0) return FLR_OK;
-    const int copies = runs_homogeneous(S, p->form, p->n_paths, p->hero) && n_film <= FILM_COPIES_MAX_VALUES ? FILM_COPIES : 1;
+    int copies = runs_homogeneous(S, p->form, p->n_paths, p->hero) && n_film <= FILM_COPIES_MAX_VALUES ? FILM_COPIES : 1;
     if (film_on) {
         rc = film_accumulator(ctx, n_film, copies, st);
         if (rc != FLR_OK) return rc;
@@ -936,7 +938,8 @@ int flr_render_camera(flr_ctx *ctx, const flr_params *p, void *stream)
         if (e != cudaSuccess) return cuda_fail(ctx, e, "clear film");
     }
     if (p->n_paths == 0) return FLR_OK;
-    rc = film_accumulator(ctx, n_film, 1, st);
+    int copies = 1;
+    rc = film_accumulator(ctx, n_film, copies, st);
     if (rc != FLR_OK) return rc;
     // the kernel's block tallies are flushed into a scratch copy: the camera estimator has none
     rc = grow(ctx, (void **)&ctx->d_adj_tal, &ctx->adj_tal_cap, (size_t)tal_size(FLR_MAX_BINS),
@@ -1278,11 +1281,19 @@ static int grow(flr_ctx *ctx, void **ptr, size_t *cap, size_t need, size_t elem,
     return FLR_OK;
 }
 
-static int film_accumulator(flr_ctx *ctx, size_t n, int copies, cudaStream_t st)
+static int film_accumulator(flr_ctx *ctx, size_t n, int &copies, cudaStream_t st)
 {
-    const int rc = grow(ctx, (void **)&ctx->d_film_fx, &ctx->film_fx_cap, film_capacity(n), sizeof(unsigned long long),
-                        "film accumulator");
-    if (rc != FLR_OK) return rc;
+    if (n > ctx->film_fx_values) {
+        void **const p = (void **)&ctx->d_film_fx;
+        int rc = grow(ctx, p, &ctx->film_fx_cap, film_capacity(n), sizeof(unsigned long long), "film accumulator");
+        if (rc == FLR_ERR_OOM && film_capacity(n) > n) {
+            (void)cudaGetLastError();   // handled here: the launches check this error word
+            rc = grow(ctx, p, &ctx->film_fx_cap, n, sizeof(unsigned long long), "film accumulator");
+        }
+        ctx->film_fx_values = rc == FLR_OK ? n : 0;
+        if (rc != FLR_OK) return rc;
+    }
+    copies = (int)std::min<size_t>(copies, ctx->film_fx_cap / n);
     const cudaError_t e = cudaMemsetAsync(ctx->d_film_fx, 0, sizeof(unsigned long long) * n * copies, st);
     return e == cudaSuccess ? FLR_OK : cuda_fail(ctx, e, "clear film accumulator");
 }

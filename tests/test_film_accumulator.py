@@ -59,3 +59,25 @@ def test_a_smaller_film_after_a_larger_one_allocates_nothing(large, small):
     finally:
         N.flr_debug_fail_alloc(0)
     S.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("film,n_paths", [(1, 2_000), (33, 2_000), (64, 1 << 22), (81, 2_000)])
+def test_a_film_whose_copies_find_no_memory_renders_with_one(film, n_paths):
+    """A launch needs one accumulator value a film value; the copies only make it faster."""
+    from paper_1706_03024_gb300.scene import Scene
+    from tests.gpu_common import require_gpu
+    require_gpu()
+    films = []
+    for fail in (0, 1):
+        S = Scene(sg.cfg1_homogeneous_cube(n_paths=n_paths, film=film))
+        S.render(form="wavefront_warp", film=False)
+        N.flr_debug_fail_alloc(fail)   # the accumulator with all its copies
+        try:
+            films.append(S.render(form="wavefront_warp").clone())
+        finally:
+            N.flr_debug_fail_alloc(0)
+        films.append(S.render(form="wavefront_warp").clone())
+        S.close()
+    assert float(films[0].sum()) > 0.0
+    assert all(bool((f == films[0]).all()) for f in films)
