@@ -840,7 +840,8 @@ int flr_render(flr_ctx *ctx, const flr_params *p, void *stream)
         ctx->paths_since_clear = 0;
     }
     if (p->n_paths == 0) return FLR_OK;
-    int copies = runs_homogeneous(S, p->form, p->n_paths, p->hero) && n_film <= FILM_COPIES_MAX_VALUES ? FILM_COPIES : 1;
+    int copies = n_film <= FILM_COPIES_MAX_VALUES ? FILM_COPIES : 1;
+    if (!runs_homogeneous(S, p->form, p->n_paths, p->hero, p->paper_mode, film_on, copies)) copies = 1;
     if (film_on) {
         rc = film_accumulator(ctx, n_film, copies, st);
         if (rc != FLR_OK) return rc;

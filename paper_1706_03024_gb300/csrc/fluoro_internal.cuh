@@ -232,8 +232,29 @@ inline size_t film_capacity(size_t n)
     const size_t with_copies = (n < FILM_COPIES_MAX_VALUES ? n : FILM_COPIES_MAX_VALUES) * FILM_COPIES;
     return n > with_copies ? n : with_copies;
 }
-// True if launch_trace runs the homogeneous medium's own kernel, which uses the copies.
-bool runs_homogeneous(const SceneDev &S, int form, uint64_t n_paths, int hero);
+// True if launch_trace runs the homogeneous medium's own kernel (k_trace_homogeneous), for a launch with a film or
+// without, whose film sums have `copies` copies (1 or 0: fp32 additions or one accumulator). Measured against
+// the queued kernel (times own / queued) over sigma_s 0.5 to 200 in the 1 cm cube, pencil beam and wide source,
+// walls, films from 16 to 512 and none, 2^20 to 2^25 paths:
+//  - It gains where most steps end in a vertex. In thin media (sigma_s 0.5, 2, and 5 with walls: 1.00 to 1.12; 10 and 12: a
+//    beam 0.54 to 0.97, a wide source 0.98 to 1.08) and with the paper's film, which most paths never reach (1.02 to 1.23),
+//    that is not so.
+//  - A lone lane connects its own vertices, so the longest path takes about a third longer, and the longest path grows
+//    with the square of the optical thickness tau where the work grows with tau: hence paths per unit of tau. With a film
+//    1 is passed at 1.2 to 1.5 million paths (tau 20), 2.5 (50), 5 (100) and 9 (200); from 2^17 tau on it is 0.77 to 0.92.
+//    Without connections it is passed before 2^14 tau (tau 200: 1.10 at 2^20, 0.99 at 2^21).
+//  - Additions to the film's hottest value bound it, which the copies relieve. Without them a pencil beam's film of
+//    81 x 81 (2^20 paths 1.16, 4,000,000 1.05) is never faster, but 1.01 at most from 2^24 on, where larger films
+//    (0.88) and wide sources (0.78) gain; fp32 additions alike (2^20 paths 1.13, 4,000,000 1.03, 20,000,000 1.01; wide 0.78).
+inline bool runs_homogeneous(const SceneDev &S, int form, uint64_t n_paths, int hero, int paper_mode, bool film, int copies)
+{
+    if (form != FLR_FORM_WAVEFRONT_WARP || hero != 0 || (paper_mode && film) || !S.homogeneous || S.iface) return false;
+    float edge = 0.0f;
+    for (int k = 0; k < 3; ++k) edge = edge < S.hi[k] - S.lo[k] ? S.hi[k] - S.lo[k] : edge;
+    const double tau = (double)S.sigma_s * edge;
+    const uint64_t least = !film ? (uint64_t)1 << 20 : copies >= FILM_COPIES ? (uint64_t)1 << 22 : (uint64_t)1 << 24;
+    return tau >= 16.0 && n_paths >= least && (double)n_paths >= (film ? 131072.0 : 16384.0) * tau;
+}
 // film[j] = fx[j] * 2^-32 (add = 0) or film[j] + fx[j] * 2^-32 (add = 1), j < n, through fp64.
 cudaError_t launch_film_fold(float *film, const unsigned long long *fx, size_t n, int copies, int add,
                              cudaStream_t st);

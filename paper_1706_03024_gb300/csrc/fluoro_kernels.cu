@@ -2856,12 +2856,10 @@ __global__ void __launch_bounds__(256) k_trace_plain(SceneDev S, RunDev R)
 // so each lane connects its vertex at once, without queues, marches or the generators they seed (71 registers,
 // seven blocks an SM). It was then bound by the film's hottest value (without film additions 13.0 ms instead of 16.7,
 // whatever the blocks), so a small film's sums are spread over FILM_COPIES copies, which the fold adds up. The
-// cube of a pencil beam, 20,000,000 paths: 17.3 -> 13.4 ms on a 64 x 64 film, 15.2 on a 256 x 256 one (no copies); 4,000,000:
-// 3.97 -> 3.38. A small launch lasts as long as its longest path, which here waits for its own connections:
-// 10,000 paths 0.41 -> 0.52 ms, 250,000 0.86 -> 1.02, 1,000,000 1.45 -> 1.47. Hence HOMOGENEOUS_MIN; below it, and
-// with interfaces, the queued kernel runs. `regroup` has no meaning here.
-constexpr unsigned long long HOMOGENEOUS_MIN = 1ull << 20;
-
+// cube of a pencil beam, 20,000,000 paths: 17.4 -> 13.3 ms on a 64 x 64 film, 15.4 on a 256 x 256 one (no copies); 4,000,000:
+// 3.87 -> 3.24. A small launch lasts as long as its longest path, which here waits for its own connections
+// (10,000 paths 0.41 -> 0.52 ms, 250,000 0.86 -> 1.02): runs_homogeneous says which launches come here; the others, and
+// those with interfaces, run the queued kernel. `regroup` has no meaning here.
 __global__ void __launch_bounds__(WARP_BLOCK, 7) k_trace_homogeneous(SceneDev S, RunDev R)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -4566,11 +4564,6 @@ cudaError_t launch_pool(const SceneDev &S, const RunDev &R, int blocks_per_sm, c
     return cudaGetLastError();
 }
 
-bool runs_homogeneous(const SceneDev &S, int form, uint64_t n_paths, int hero)
-{
-    return form == FLR_FORM_WAVEFRONT_WARP && hero == 0 && S.homogeneous && !S.iface && n_paths >= HOMOGENEOUS_MIN;
-}
-
 cudaError_t launch_homogeneous(const SceneDev &S, const RunDev &R, int block, int blocks_per_sm, cudaStream_t st)
 {
     block = block <= 0 ? WARP_BLOCK : std::min(block, WARP_BLOCK);
@@ -4589,7 +4582,8 @@ cudaError_t launch_trace(const SceneDev &S, const RunDev &R, int form, int block
 {
     if (form == FLR_FORM_WAVEFRONT_POOL) return launch_pool(S, R, blocks_per_sm, st);
     if (R.hero > 0 && form == FLR_FORM_WAVEFRONT_WARP) return launch_hero_warp(S, R, block, blocks_per_sm, st);
-    if (runs_homogeneous(S, form, R.n_paths, R.hero)) return launch_homogeneous(S, R, block, blocks_per_sm, st);
+    if (runs_homogeneous(S, form, R.n_paths, R.hero, R.paper_mode, R.film != nullptr, R.film_copies))
+        return launch_homogeneous(S, R, block, blocks_per_sm, st);
     if (block <= 0) block = trace_block_default();
     if (form == FLR_FORM_WAVEFRONT_WARP) block = std::min(block, WARP_BLOCK);
     const int smem = trace_smem_bytes(S.B, form, block);
