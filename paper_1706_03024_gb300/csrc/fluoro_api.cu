@@ -235,6 +235,15 @@ void build_tables(flr_ctx *ctx)
                         ctx->tables_margin);
 }
 
+// A component of a caller's direction. The kernels work with its reciprocal times box and cell edges, which has to be a
+// finite number: 0 x infinity would lose the order of the cells along a ray. So components under 2^-100 are raised to
+// it, keeping their sign; no ray inside a box moves by that much.
+float direction_component(float v)
+{
+    constexpr float least = 0x1p-100f;
+    return v != 0.0f && std::fabs(v) < least ? std::copysign(least, v) : v;
+}
+
 // The spectral lines of a medium's sources, chosen in proportion to power (p(lambda_x), Eq. 12).
 int build_emitters(flr_ctx *ctx, const flr_medium &m, int max_lines, EmitterDev *em, float *em_cdf,
                    int *n_out, int *group_first = nullptr, int *group_n = nullptr)
@@ -257,7 +266,7 @@ int build_emitters(flr_ctx *ctx, const flr_medium &m, int max_lines, EmitterDev 
                 e.origin[k] = src.origin[k];
                 e.eu[k] = src.eu[k];
                 e.ev[k] = src.ev[k];
-                e.dir[k] = src.dir[k];
+                e.dir[k] = direction_component(src.dir[k]);
             }
             e.kind = src.kind;
             e.bin = snap_bin(src.lambda_nm[l], ctx->lambda0, ctx->dlambda, ctx->B);
@@ -368,7 +377,7 @@ int fill_scene(flr_ctx *ctx, SceneDev &S, bool with_film, int macro_cell = 0, in
         S.H = c.height;
         for (int k = 0; k < 3; ++k) {
             S.s_origin[k] = c.origin[k];
-            S.s_view[k] = c.view[k];
+            S.s_view[k] = direction_component(c.view[k]);
         }
         if (c.kind == FLR_SENSOR_ORTHO) {
             double uu = 0, vv = 0;
