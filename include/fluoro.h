@@ -172,7 +172,9 @@ typedef struct flr_params {
     int block_size;              /* threads per block; 0 = library default (the warp-regrouped
                                     form and the adjoint's passes use at most 128)              */
     int blocks_per_sm;           /* resident blocks per SM; 0 = occupancy maximum               */
-    int regroup_interval;        /* wavefront: tracking steps between connection flushes; 0 auto */
+    int regroup_interval;        /* wavefront, wavefront_warp: tracking steps a lane makes between two looks
+                                    at its queue; 0 auto (8, 1), above 64 as 64; without effect on the
+                                    results, and on large launches of homogeneous media */
     int macro_cell;              /* > 0: free flights and transmittance marches use local
                                     majorants over cells of macro_cell^3 voxels (each the maximum
                                     of sigma_t over the cell and a one-voxel halo), walked by DDA;

@@ -489,7 +489,8 @@ __device__ __forceinline__ float sqrt_approx(float x)
 
 // The hardware's approximate reciprocal (PTX rcp.approx.ftz.f32, 1 ulp). The same bits as
 // __fdividef(1, x) for every normal x whose reciprocal is normal, without the range checks that
-// surround it (3 instructions instead of 10).
+// surround it (3 instructions instead of 10). Subnormal x give infinity: the host keeps them out of
+// directions (direction_component).
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float r;
@@ -1323,14 +1324,13 @@ __device__ __forceinline__ Conn track_body(const M &m, const RunDev &R, const Sm
 }
 
 // The step with its end: the count and the path's event record stand once, behind the step, instead
-// of at each of the fourteen places where a path can end. What bounds the persistent kernels is the
-// instruction cache: at five warps a scheduler more warps only raise the stalls for want of an
-// instruction (0.55 to 3.6 per instruction at eight), and a kernel of more phases than tracking and
-// drain loses more to them than its fuller lanes gain. So the loops' code is kept small: this, the
-// counters of cnt_add, the selects of exit_distance and the reciprocals of inv_dir took the step
-// from 1,460 to 860 instructions, and (per call, on the current sizes) the Cornell box from 11.07 to
+// of at each of the fourteen places where a path can end. The loops' code is kept small: the warp kernels wait 0.4
+// cycles an issued instruction for want of an instruction, the hero kernel waited 1.0 with 71 KB of code (63 now) and 2.1
+// with its spawns in the step. This, the counters of cnt_add, the selects of exit_distance and the reciprocals of inv_dir took the step
+// from 1,460 to 860 instructions, and (per call, each against the sources before it) the Cornell box from 11.07 to
 // 10.08 ms, with four hero wavelengths (8 paths a pixel) from 11.31 to 8.58 ms, the light sheet from 205 to
-// 189 ms, 256 batched media from 41.3 to 37.8 ms, the camera view from 0.84 to 0.76 ms.
+// 189 ms, the camera view from 0.84 to 0.76 ms; 256 batched media, whose kernel was bounded to 64 registers in the same
+// step, from 41.3 to 37.8 ms.
 template <class M, class Obs = NoObs>
 __device__ __forceinline__ Conn track_step(const M &m, const RunDev &R, const Smem &sm, Path &p,
                                            RegCnt &rc, const Obs &obs = Obs())
@@ -1444,9 +1444,11 @@ constexpr int WQ_CAP = 128;
 constexpr int WQ_DRAIN = WQ_CAP - 32;
 constexpr int MS_CAP = 64;        // stack of marches that wait: fewer than 32 before 32 records are begun
 constexpr int MS_WORDS = 19;      // 4-byte fields per waiting march
-constexpr int DRAIN_KEEP = 16;    // a drain ends once fewer lanes would go on (24: 226 for 229 ms on the sheet, more on the box)
+constexpr int DRAIN_KEEP = 16;    // a drain ends once fewer lanes would go on (8 / 16 / 24: the light sheet 174.9 / 169.9 / 167.9 ms,
+                                  // the Cornell box 10.99 / 10.53 / 10.35, the vial 1.02 / 1.00 / 0.99: more than 16 would be faster)
 constexpr int SPAWN_MIN = 8;      // lanes that start new paths together (hero, camera; pass 2 of the adjoint)
-constexpr int CLAIM_MIN = 4;      // lanes that take path ids together (the light sheet: 1: 180, 4: 182, 8: 189 ms)
+constexpr int CLAIM_MIN = 4;      // lanes that take path ids together (1 / 4 / 8: the light sheet 169.4 / 169.9 / 177.0 ms, the Cornell
+                                  // box 10.56 / 10.53 / 10.72, the vial 1.011 / 0.997 / 1.000, a fit's step 16.89 / 16.79 / 17.02)
 constexpr int WARP_WORDS = 6;     // head, tail and PathIds of a warp (8-byte aligned)
 static_assert(WQ_DRAIN + 31 < WQ_CAP, "warp queue overflow");
 static_assert(MS_CAP >= 64 && DRAIN_KEEP <= 32, "march stack overflow");
@@ -2388,13 +2390,12 @@ __global__ void __launch_bounds__(256) k_frozen_sums(SceneDev S, RunDev R, PertD
 }
 
 // ---------------------------------------------------------------------------------------------
-// Wavefront form with per-warp regrouping and pull-based connection drains. Each warp queues its
-// lanes' sensor connections in shared memory (up to WQ_CAP records). Once WQ_DRAIN records are
-// waiting (or the work is done) the warp drains the queue: every lane advances its own
-// ratio-tracking march by one step per iteration and claims the next record as soon as its march
-// ends, so the lanes stay busy until the queue runs dry instead of waiting for the longest march
-// of a fixed batch. The marches consume their random numbers exactly as transmittance() does, so
-// every launch form gives the same film up to the order of the fp32 film atomics.
+// Wavefront form with per-warp regrouping. Each warp queues its lanes' sensor connections in shared memory
+// (up to WQ_CAP records). Once WQ_DRAIN records are waiting, or the work is done, it drains them (wq_drain):
+// records are begun 32 together, what is left of them waits on a stack, and each lane advances one ratio-tracking
+// march a step an iteration and takes the next from the stack as soon as its march ends; the last few marches
+// go back to the stack for the next drain. The marches consume their random numbers exactly as
+// transmittance() does and the film's sums are exact, so every launch form gives the same film bit for bit.
 //
 // The same kernel runs the two passes of the adjoint replay (MODE):
 //   WM_RENDER       film contributions (the forward);
@@ -3336,7 +3337,8 @@ __global__ void __launch_bounds__(WARP_BLOCK, 5) k_trace_pool(SceneDev S, RunDev
         }
         const int avail = q.head_tail[1];
         if (avail >= PQ_DRAIN || (kind == 3 && avail > 0)) {
-            // pull-based drain of all `avail` records (as in k_trace_wavefront_warp)
+            // pull-based drain of all `avail` records: a lane whose march ended claims the next record in the
+            // next iteration
             March mc;
             bool active = false;
             int claimed = 0;
@@ -3366,12 +3368,11 @@ __global__ void __launch_bounds__(WARP_BLOCK, 5) k_trace_pool(SceneDev S, RunDev
 }
 
 // ---------------------------------------------------------------------------------------------
-// Warp-regrouped form of the hero-wavelength tracer: the tracking round and the pull-based drains
-// of k_trace_wavefront_warp, with records that carry the member set. A record holds the vertex, the
+// Warp-regrouped form of the hero-wavelength tracer: per-warp queues with pull-based drains (a lane whose march
+// ended claims the next record), with records that carry the member set. A record holds the vertex, the
 // path weight, the members' weights q_j and packed bins, the member count, the hero's index and the
 // vertex kind, and the RNG coordinates (13 words). A drain's march estimates every member's
-// transmittance at once (connect_hero's march, step by step), so the film matches the plain hero
-// form's up to the order of the fp32 atomics.
+// transmittance at once (connect_hero's march, step by step), so the film is the plain hero form's bit for bit.
 constexpr int HQ_CAP = 224;
 constexpr int HQ_DRAIN = 192;
 constexpr int HQ_WORDS = 13;
@@ -3936,9 +3937,8 @@ __global__ void __launch_bounds__(256) k_trace_camera(SceneDev S, RunDev R)
 }
 
 // Warp-regrouped form: the lanes' light samples go to a per-warp shared-memory queue and are
-// marched by whole warps, one march per lane, with pull-based claims as in the light tracer's warp
-// form. The marches draw the same uniforms as transmittance(), so both forms give the same film up
-// to the order of fp32 additions.
+// marched by whole warps, one march per lane, with pull-based claims. The marches draw the same uniforms as
+// transmittance() and the film's sums are exact, so both forms give the same film bit for bit.
 constexpr int CQ_CAP = 160;
 constexpr int CQ_DRAIN = 128;
 constexpr int CQ_WORDS = 13;   // start 3, dir 3, len, weight, pixel, bins, pid lo/hi, step
@@ -4024,7 +4024,7 @@ __global__ void __launch_bounds__(256, 2) k_trace_camera_warp(SceneDev S, RunDev
         const int avail = queue_length(tail);
         const bool any = __any_sync(FULL, cp.alive || !exhausted);
         if (avail >= CQ_DRAIN || (!any && avail > 0)) {
-            // pull-based drain; claims every second iteration (see the light tracer's warp form)
+            // pull-based drain: a lane whose march ended claims the next record in the next iteration
             float3 x0, dir;
             float tl = 0.0f, t = 0.0f, T = 1.0f, isb = 0.0f, wt = 0.0f;
             int pix = 0, bin = 0, bx = 0, it = 0;
