@@ -2854,7 +2854,7 @@ __global__ void __launch_bounds__(256) k_trace_plain(SceneDev S, RunDev R)
 // ---------------------------------------------------------------------------------------------
 // The warp form of a homogeneous medium with index-matched faces and Lambertian walls. There nearly every
 // step of a lane ends in a vertex, and a vertex's transmittance is closed (Eq. 6): nothing is to be regrouped,
-// so each lane connects its vertex at once, without queues, marches or the generators they seed (71 registers,
+// so each lane connects its vertex at once, without queues, marches or the generators they seed (70 registers,
 // seven blocks an SM). It was then bound by the film's hottest value (without film additions 13.0 ms instead of 16.7,
 // whatever the blocks), so a small film's sums are spread over FILM_COPIES copies, which the fold adds up. The
 // cube of a pencil beam, 20,000,000 paths: 17.4 -> 13.3 ms on a 64 x 64 film, 15.4 on a 256 x 256 one (no copies); 4,000,000:
